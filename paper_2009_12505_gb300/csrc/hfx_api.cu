@@ -1984,10 +1984,15 @@ hfx_status hfx_stats(const hfx_ctx *ctx, void *stats) {
 // ------------------------------------------------- steps next to the build
 
 namespace {
+// No early exit, so that the loop vectorises.
 bool finite_all(const double *x, int64_t n) {
-  for (int64_t i = 0; i < n; ++i)
-    if (!std::isfinite(x[i])) return false;
-  return true;
+  uint64_t bad = 0;
+  for (int64_t i = 0; i < n; ++i) {
+    uint64_t b;
+    std::memcpy(&b, x + i, sizeof(b));
+    bad |= (b & 0x7FF0000000000000ull) == 0x7FF0000000000000ull;
+  }
+  return bad == 0;
 }
 }  // namespace
 
@@ -2018,32 +2023,54 @@ hfx_status hfx_density_from_eigvecs(hfx_ctx *ctx, int32_t nk, const double *kfra
     if (max_imag) *max_imag = 0.0;
     return HFX_OK;
   }
+  // keys grouped by unordered atom pair, at most DENSITY_IMAGES to a group: the
+  // pair's band sums are formed once for all of them.  A key (i, j, n) with
+  // i > j is the conjugate transpose of the pair (j, i) turned by its own phase
+  std::vector<int64_t> order(nkeys);
+  for (int64_t e = 0; e < nkeys; ++e) order[e] = e;
+  auto pair_of = [&](int64_t e) {
+    const int32_t *k = keys + 5 * e;
+    return ((uint64_t)std::min(k[0], k[1]) << 32) | (uint32_t)std::max(k[0], k[1]);
+  };
+  std::stable_sort(order.begin(), order.end(),
+                   [&](int64_t x, int64_t y) { return pair_of(x) < pair_of(y); });
+  std::vector<DensityKey> hk(nkeys);
+  std::vector<DensityGroup> hg;
+  for (int64_t q = 0; q < nkeys; ++q) {
+    const int32_t *k = keys + 5 * order[q];
+    hk[q] = DensityKey{{k[2], k[3], k[4]}, k[0] > k[1] ? 1 : 0, doff[order[q]]};
+    const int32_t K = std::min(k[0], k[1]), L = std::max(k[0], k[1]);
+    if (hg.empty() || hg.back().K != K || hg.back().L != L || hg.back().count == DENSITY_IMAGES)
+      hg.push_back(DensityGroup{K, L, (int32_t)q, 0});
+    ++hg.back().count;
+  }
   cudaStream_t st = ctx->stream;
   DevBuf<double> dk, dc, dq, dout;
-  DevBuf<int32_t> dkeys, daoff, dnao;
-  DevBuf<int64_t> ddoff;
+  DevBuf<int32_t> daoff, dnao;
+  DevBuf<DensityKey> dkeys;
+  DevBuf<DensityGroup> dgroups;
   DevBuf<unsigned long long> dmax;
   CK(dk.reserve(3 * nk));
   CK(dc.reserve(ncoef));
   CK(dq.reserve(nocc));
   CK(dout.reserve(doff[nkeys]));
-  CK(dkeys.reserve(5 * nkeys));
+  CK(dkeys.reserve(nkeys));
+  CK(dgroups.reserve(hg.size()));
   CK(daoff.reserve(natoms + 1));
   CK(dnao.reserve(natoms));
-  CK(ddoff.reserve(nkeys + 1));
   CK(dmax.reserve(1));
   CK(cudaMemcpyAsync(dk.p, kfrac, sizeof(double) * 3 * nk, cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(dc.p, coef, sizeof(double) * ncoef, cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(dq.p, occ, sizeof(double) * nocc, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(dkeys.p, keys, sizeof(int32_t) * 5 * nkeys, cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(dkeys.p, hk.data(), sizeof(DensityKey) * nkeys, cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(dgroups.p, hg.data(), sizeof(DensityGroup) * hg.size(),
+                     cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(daoff.p, aoff.data(), sizeof(int32_t) * (natoms + 1), cudaMemcpyHostToDevice,
                      st));
   CK(cudaMemcpyAsync(dnao.p, ctx->nao.data(), sizeof(int32_t) * natoms, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(ddoff.p, doff.data(), sizeof(int64_t) * (nkeys + 1), cudaMemcpyHostToDevice,
-                     st));
   CK(cudaMemsetAsync(dmax.p, 0, sizeof(unsigned long long), st));
-  CK(launch_density(nk, dk.p, (int)nb, nbands, dc.p, dq.p, nkeys, dkeys.p, daoff.p, dnao.p,
-                    ddoff.p, dout.p, dmax.p, st));
+  CK(launch_density(nk, dk.p, (int)nb, nbands, dc.p, dq.p, (int64_t)hg.size(), dgroups.p, dkeys.p,
+                    daoff.p, dnao.p, dout.p, dmax.p, st));
   unsigned long long mbits = 0;
   CK(cudaMemcpyAsync(out, dout.p, sizeof(double) * doff[nkeys], cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(&mbits, dmax.p, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));

@@ -209,9 +209,21 @@ cudaError_t launch_check_mirror(const double *data, const int64_t *offs, const i
 cudaError_t launch_gather(const double *const *src, const int64_t *dst_off, const int64_t *len,
                           int64_t nblk, double *dst, cudaStream_t st);
 // Density-matrix blocks from eigenvectors and Sigma at k points (hfx_fourier.cu).
+// One density key of a group: its lattice vector, whether its block is (L, K)
+// for the group's pair (K, L), and the offset of its block in the output.
+struct DensityKey {
+  int32_t n[3];
+  int32_t tr;
+  int64_t off;
+};
+// Keys [first, first + count) of the atom pair (K, L), count <= DENSITY_IMAGES.
+constexpr int DENSITY_IMAGES = 8;
+struct DensityGroup {
+  int32_t K, L, first, count;
+};
 cudaError_t launch_density(int nk, const double *kfrac, int nb, int nbands, const double *coef,
-                           const double *occ, int64_t nkeys, const int32_t *keys,
-                           const int32_t *aoff, const int32_t *nao, const int64_t *doff,
+                           const double *occ, int64_t ngroups, const DensityGroup *groups,
+                           const DensityKey *dkeys, const int32_t *aoff, const int32_t *nao,
                            double *out, unsigned long long *maxim, cudaStream_t st);
 cudaError_t launch_sigma_k(int nk, const double *kfrac, int natoms, const int32_t *aoff,
                            const int32_t *nao, int64_t nkeys, const uint64_t *skeys,

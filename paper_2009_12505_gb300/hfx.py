@@ -354,16 +354,16 @@ class Context:
         fractional k points kfrac (nk, 3).  Returns (packed blocks in key
         order, largest |imaginary part| dropped)."""
         kf = np.ascontiguousarray(np.asarray(kfrac, np.float64).reshape(-1, 3))
-        c = np.asarray(coef, np.complex128)
-        nk, nbasis, nbands = c.shape
-        cc = np.ascontiguousarray(np.stack([c.real, c.imag], axis=-1))
+        cc = np.ascontiguousarray(coef, np.complex128)  # (re, im) pairs as they lie
+        nk, nbasis, nbands = cc.shape
         f = np.ascontiguousarray(np.asarray(occ, np.float64).reshape(nk, nbands))
         k = np.ascontiguousarray(np.asarray(keys, np.int32).reshape(-1, 5))
         nat = len(self.nao)
         ok = (k[:, 0] >= 0) & (k[:, 0] < nat) & (k[:, 1] >= 0) & (k[:, 1] < nat)
         # keys with atoms out of range are rejected by the library (HFX_E_ARG)
-        size = int(sum(int(self.nao[a]) * int(self.nao[b]) for a, b in k[ok][:, :2].tolist()))
-        out = np.zeros(max(size, 1), np.float64)
+        nao = self.nao.astype(np.int64)
+        size = int((nao[k[ok, 0]] * nao[k[ok, 1]]).sum())
+        out = np.empty(max(size, 1), np.float64)
         mi = ctypes.c_double(0.0)
         self._check(self._lib.hfx_density_from_eigvecs(self._h, nk, _p(kf), nbands, _p(cc), _p(f),
                                                         k.shape[0], _p(k), _p(out),
@@ -374,9 +374,9 @@ class Context:
         """The last build's Sigma at fractional k points: complex (nk, nb, nb)."""
         kf = np.ascontiguousarray(np.asarray(kfrac, np.float64).reshape(-1, 3))
         nb = int(np.sum(self.nao))
-        out = np.zeros((kf.shape[0], nb, nb, 2), np.float64)
+        out = np.empty((kf.shape[0], nb, nb), np.complex128)
         self._check(self._lib.hfx_sigma_k(self._h, kf.shape[0], _p(kf), _p(out)))
-        return out[..., 0] + 1j * out[..., 1]
+        return out
 
     def stats(self) -> dict:
         s = Stats()
