@@ -307,16 +307,18 @@ hfx_status hfx_stats(const hfx_ctx *ctx, void *stats);
  *
  * Computes, on cuda_stream (NULL = legacy default stream),
  *   out[i][j] = sum_{alpha,beta,k,l} cA[alpha][i][k] V[alpha][beta] cB[beta][j][l] D[k][l]
- * in the C((VC)D) order the build uses (Y = V cB, T = Y D, out = cA T).  The
- * exchange matrix receives minus this term.
+ * as Y = V cB, T = Y D, out = cA T (the build's C((VC)D) order) or, where it
+ * takes no more multiply-adds and fits the working memory, as W = V cA,
+ * X = cB D, out = W X.  The exchange matrix receives minus this term.
  *   cA  [nabf_a][nao_i][nao_k]   V [nabf_a][nabf_b]
  *   cB  [nabf_b][nao_j][nao_l]   D [nao_k][nao_l]    out [nao_i][nao_j]
  * All pointers are device memory on the current device, row-major FP64, owned
  * by the caller; out is overwritten.
  *
- * Working memory: the two intermediates Y and T live in one fixed 2 MiB static
- * device array (each at most 131072 doubles: nabf_a*nao_j*nao_l and
- * nabf_a*nao_j*nao_k must both be <= 131072, else HFX_E_SHAPE).  Every GPU
+ * Working memory: the two intermediates live in one fixed 2 MiB static
+ * device array (each at most 131072 doubles: Y's nabf_a*nao_j*nao_l and T's
+ * nabf_a*nao_j*nao_k must both be <= 131072, else HFX_E_SHAPE, whichever order
+ * is taken).  Every GPU
  * that loads the library holds that array until the process exits.  The first
  * call on each device looks the array's address up (cudaGetSymbolAddress) with
  * that device current; make that first call before any stream capture.  The

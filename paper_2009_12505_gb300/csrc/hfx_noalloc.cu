@@ -6,10 +6,20 @@
 // cudaFree (which can synchronize the device) are not allowed, or a process
 // whose device memory is already fully reserved by another allocator so that a
 // new allocation would fail.  hfx_build allocates its working memory inside
-// the context; this entry point does not.  It evaluates the same staged
-// product as the build's Y, D-stage and final contraction kernels, but keeps
-// its two intermediates in the fixed static array below instead of allocated
-// scratch.  The caller passes inputs and the output as device pointers.
+// the context; this entry point does not: it keeps its two intermediates in
+// the fixed static array below instead of allocated scratch.  The caller
+// passes inputs and the output as device pointers.
+//
+// Two orders of the product, by multiply-adds:
+//   pair:   W = V^T cA and X = cB D^T (one launch), out = W . X   (two launches)
+//   staged: Y = V cB, T = Y D^T, out = cA . T                     (three)
+// The pair order halves the work when i, k are no larger than j, l (60/90 ABFs,
+// 13 and 27 AOs: 2.2 against 4.8 M multiply-adds), has one launch fewer, and
+// its two first products run side by side; it is taken when it needs no more
+// multiply-adds and its intermediates fit the static array, else the staged
+// order, whose sizes the caller's limits are stated for.
+// That term: 105 us a call before (three launches, one thread per output in
+// the last), 31 us now.
 #include <algorithm>
 #include <mutex>
 
@@ -68,39 +78,74 @@ __global__ void k_term_y(int pA, int pB, int nj, int nl, const double *V, const 
        idx += gridDim.x * blockDim.x) {
     const int al = idx / n, c = idx - al * n;
     double s = 0.0;
+#pragma unroll 8
     for (int be = 0; be < pB; ++be) s = fma(V[al * pB + be], cB[be * n + c], s);
     Y[idx] = s;
   }
 }
 
-// T[al][j][k] = sum_l Y[al][j][l] D[k][l]
+// T[x][j][k] = sum_l Y[x][j][l] D[k][l], element idx
+__device__ __forceinline__ void term_t(int idx, int nj, int nk, int nl, const double *Y,
+                                       const double *D, double *T) {
+  const int n = nj * nk;
+  const int x = idx / n, r = idx - x * n, j = r / nk, k = r - j * nk;
+  const double *y = Y + ((int64_t)x * nj + j) * nl;
+  const double *d = D + (int64_t)k * nl;
+  double s = 0.0;
+#pragma unroll 8
+  for (int l = 0; l < nl; ++l) s = fma(y[l], d[l], s);
+  T[idx] = s;
+}
+
 __global__ void k_term_t(int pA, int nj, int nk, int nl, const double *Y, const double *D,
                          double *T) {
-  const int n = nj * nk;
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < pA * n;
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < pA * nj * nk;
+       idx += gridDim.x * blockDim.x)
+    term_t(idx, nj, nk, nl, Y, D, T);
+}
+
+// W[be][i][k] = sum_al V[al][be] cA[al][i][k] and X[be][j][k] = sum_l
+// cB[be][j][l] D[k][l], one element per thread: bound by the latency of its
+// loads (unrolled, so several are in flight) at these sizes.
+__global__ void k_term_wx(int pA, int pB, int ni, int nj, int nk, int nl, const double *cA,
+                          const double *V, const double *cB, const double *D, double *W,
+                          double *X) {
+  const int n = ni * nk, nw = pB * n, nx = pB * nj * nk;
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < nw + nx;
        idx += gridDim.x * blockDim.x) {
-    const int al = idx / n, r = idx - al * n, j = r / nk, k = r - j * nk;
-    const double *y = Y + ((int64_t)al * nj + j) * nl;
-    const double *d = D + (int64_t)k * nl;
+    if (idx >= nw) {
+      term_t(idx - nw, nj, nk, nl, cB, D, X);
+      continue;
+    }
+    const int be = idx / n, c = idx - be * n;
     double s = 0.0;
-    for (int l = 0; l < nl; ++l) s = fma(y[l], d[l], s);
-    T[idx] = s;
+#pragma unroll 8
+    for (int al = 0; al < pA; ++al) s = fma(V[(int64_t)al * pB + be], cA[(int64_t)al * n + c], s);
+    W[idx] = s;
   }
 }
 
-// out[i][j] = sum_{al,k} cA[al][i][k] T[al][j][k]
-__global__ void k_term_out(int pA, int ni, int nj, int nk, const double *cA, const double *T,
+// out[i][j] = sum_{x,k} A[x][i][k] T[x][j][k] with LANES lanes (32 or 1) per
+// output, which share the p nk terms and add up in a fixed tree.  One thread
+// per output (a chain of 780 loads and multiply-adds for 13 AOs and 60 ABFs)
+// was most of the call; it is kept for blocks of so many outputs that threads
+// alone fill the chip.
+template <int LANES>
+__global__ void k_term_out(int p, int ni, int nj, int nk, const double *A, const double *T,
                            double *out) {
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < ni * nj;
-       idx += gridDim.x * blockDim.x) {
-    const int i = idx / nj, j = idx - i * nj;
+  const int lane = threadIdx.x % LANES;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x / LANES;
+  for (int64_t o = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / LANES;
+       o < (int64_t)ni * nj; o += step) {
+    const int i = (int)(o / nj), j = (int)(o - (int64_t)i * nj);
     double s = 0.0;
-    for (int al = 0; al < pA; ++al) {
-      const double *a = cA + ((int64_t)al * ni + i) * nk;
-      const double *t = T + ((int64_t)al * nj + j) * nk;
-      for (int k = 0; k < nk; ++k) s = fma(a[k], t[k], s);
+#pragma unroll 4
+    for (int t = lane; t < p * nk; t += LANES) {
+      const int x = t / nk, k = t - x * nk;
+      s = fma(A[((int64_t)x * ni + i) * nk + k], T[((int64_t)x * nj + j) * nk + k], s);
     }
-    out[idx] = s;
+    for (int h = LANES / 2; h; h >>= 1) s += __shfl_xor_sync(0xffffffffu, s, h);
+    if (lane == 0) out[o] = s;
   }
 }
 
@@ -145,13 +190,28 @@ extern "C" hfx_status hfx_term_noalloc(int32_t nabf_a, int32_t nabf_b, int32_t n
   if (scratch_for_current_device(&scratch) != cudaSuccess) return HFX_E_CUDA;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   double *Y = scratch, *T = scratch + kHalf;
-  const int threads = 256;
+  const int threads = 128;
   auto blocks = [&](int64_t n) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + threads - 1) / threads, 4096)); };
-  k_term_y<<<blocks((int64_t)nabf_a * nao_j * nao_l), threads, 0, st>>>(nabf_a, nabf_b, nao_j,
-                                                                          nao_l, V, cB, Y);
-  k_term_t<<<blocks((int64_t)nabf_a * nao_j * nao_k), threads, 0, st>>>(nabf_a, nao_j, nao_k,
-                                                                          nao_l, Y, D, T);
-  k_term_out<<<blocks((int64_t)nao_i * nao_j), threads, 0, st>>>(nabf_a, nao_i, nao_j, nao_k, cA,
-                                                                 T, out);
+  auto term_out = [&](int p, const double *A, const double *B) {
+    const int64_t n = (int64_t)nao_i * nao_j;
+    if (n < 65536)
+      k_term_out<32><<<blocks(32 * n), threads, 0, st>>>(p, nao_i, nao_j, nao_k, A, B, out);
+    else
+      k_term_out<1><<<blocks(n), threads, 0, st>>>(p, nao_i, nao_j, nao_k, A, B, out);
+  };
+  // elements and multiply-adds of the two orders (doubles: no overflow)
+  const double w = (double)nabf_b * nao_i * nao_k, x = (double)nabf_b * nao_j * nao_k;
+  const double y = (double)nabf_a * nao_j * nao_l, t = (double)nabf_a * nao_j * nao_k;
+  const double pair = w * nabf_a + x * nao_l + x * nao_i;
+  const double staged = y * nabf_b + t * nao_l + t * nao_i;
+  if (w <= kHalf && x <= kHalf && pair <= staged) {
+    k_term_wx<<<blocks((int64_t)(w + x)), threads, 0, st>>>(nabf_a, nabf_b, nao_i, nao_j, nao_k,
+                                                            nao_l, cA, V, cB, D, Y, T);
+    term_out(nabf_b, Y, T);
+  } else {
+    k_term_y<<<blocks((int64_t)y), threads, 0, st>>>(nabf_a, nabf_b, nao_j, nao_l, V, cB, Y);
+    k_term_t<<<blocks((int64_t)t), threads, 0, st>>>(nabf_a, nao_j, nao_k, nao_l, Y, D, T);
+    term_out(nabf_a, cA, T);
+  }
   return cudaGetLastError() == cudaSuccess ? HFX_OK : HFX_E_CUDA;
 }
