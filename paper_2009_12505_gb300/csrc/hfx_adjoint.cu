@@ -18,12 +18,69 @@
 //                           + sum_b D_FB[f][b] sum_G w23 sum_g D_AG[a][g] Y[al][b][g] )
 // (C in the A role).  dC accumulates through the fixed-point adder, so the
 // gradient is bitwise reproducible; each pair owns its V block.
+//
+// FP64 runs at 1/64 of the FP32 rate here, so these kernels are bound by their
+// multiply-adds, and what saves time is not doing them:
+//  * the inner sums of Z2 and of the D_AG part of dC_AF do not depend on the
+//    other neighbour: Q_F = C_AF D_FB and T3_G = Y_G D_AG^T are formed once per
+//    pair, and the sums over F (G) add them under their weights (one add where
+//    13 multiply-adds stood);
+//  * for exactly Hermitian V and D (A.sym) the A-role gradient of <A,B> is the
+//    B-role gradient of the mirror pair <B,A> (the same quadruples with the
+//    same screen), so the B role is taken twice, neither Y nor the A role is
+//    computed, and dV is computed for one pair of two mirrors and written to
+//    both.
+// 8-atom Si-like cell, cutoffs 8 / 10 / 8 bohr: adjoint kernels 35 ms before.
 #include "fp64_common.cuh"
 
 namespace {
 
 __device__ inline int64_t dblock(const ContractArgs &A, int i, int j, int n0, int n1, int n2) {
   return dh_find(A.dhash, hk_pack(i, j, n0, n1, n2));
+}
+
+// Q_F[al][a][b] = sum_f C_AF[al][a][f] D_FB[f][b] for the F of D_FB / D_AG terms.
+__global__ void __launch_bounds__(kThreads) k_adj_q(ContractArgs A) {
+  const PairLoc L = locate(A, blockIdx.x, false);
+  const WorkItem it = A.items[L.w];
+  if (!(A.wf_flags[it.wf_off + L.idx] & 6u)) return;
+  const NbrEntry ef = A.nbr[it.fbase + L.idx];
+  const int64_t dfb = dblock(A, ef.other, it.b, it.n[0] - ef.n[0], it.n[1] - ef.n[1],
+                             it.n[2] - ef.n[2]);
+  if (dfb < 0) return;  // never read: its weight meets no D block
+  const int pA = A.nabf[it.a], na = A.nao[it.a], nb = A.nao[it.b], nf = A.nao[ef.other];
+  const double *d = A.D.data + A.D.offs[dfb], *C = A.C.data + A.C.offs[ef.cblk];
+  const int per = na * nb;
+  double *Q = A.scratch + A.q_off[L.w - A.w0] + (int64_t)L.idx * pA * per;
+  for (int idx = threadIdx.x; idx < pA * per; idx += kThreads) {
+    const int x = idx / nb, b = idx - x * nb;  // x = al na + a
+    double s = 0.0;
+    for (int f = 0; f < nf; ++f) s = fma(C[(int64_t)x * nf + f], d[f * nb + b], s);
+    Q[idx] = s;
+  }
+}
+
+// T3_G[al][a][b] = sum_g D_AG[a][g] Y[al][b][(G,g)] for the G of D_FB / D_AG terms.
+__global__ void __launch_bounds__(kThreads) k_adj_t3(ContractArgs A) {
+  const PairLoc L = locate(A, blockIdx.x, true);
+  const WorkItem it = A.items[L.w];
+  if (!(A.wg_flags[it.wg_off + L.idx] & 6u)) return;
+  const NbrEntry eg = A.nbr[it.gbase + L.idx];
+  const int64_t dag = dblock(A, it.a, eg.other, it.n[0] + eg.n[0], it.n[1] + eg.n[1],
+                             it.n[2] + eg.n[2]);
+  if (dag < 0) return;
+  const int pA = A.nabf[it.a], na = A.nao[it.a], nb = A.nao[it.b], ng = A.nao[eg.other];
+  const int ncol = A.ncol[it.b], per = na * nb;
+  const double *d = A.D.data + A.D.offs[dag];
+  const double *Y = A.scratch + A.y_off[L.w - A.w0] + eg.aopre;
+  double *T3 = A.scratch + A.t3_off[L.w - A.w0] + (int64_t)L.idx * pA * per;
+  for (int idx = threadIdx.x; idx < pA * per; idx += kThreads) {
+    const int al = idx / per, r = idx - al * per, a = r / nb, b = r - a * nb;
+    const double *y = Y + ((int64_t)al * nb + b) * ncol;
+    double s = 0.0;
+    for (int g = 0; g < ng; ++g) s = fma(d[a * ng + g], y[g], s);
+    T3[idx] = s;
+  }
 }
 
 // R[al][b][(G,g)] for one (pair, G), written over Y's layout in the R region.
@@ -67,6 +124,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_r(ContractArgs A) {
   const double *Dab = use14 ? A.D.data + A.D.offs[it.dab] : nullptr;
   const double *Dag = use23 ? A.D.data + A.D.offs[dAG] : nullptr;
   double *R = A.scratch + A.p_off[L.w - A.w0] + eg.aopre;  // R[al][b][ncol]
+  const double *Q = A.scratch + A.q_off[L.w - A.w0];
   const int per1 = na * ng, per2 = na * nb;
   const int ach = max(1, min(pA, (kChunk / 2) / max(per1, per2)));
   unsigned long long macs = 0;
@@ -89,19 +147,12 @@ __global__ void __launch_bounds__(kThreads) k_adj_r(ContractArgs A) {
       Z1[idx] = s;
     }
     for (int idx = threadIdx.x; idx < ac * per2; idx += kThreads) {
-      const int al = idx / per2, r = idx - al * per2, a = r / nb, b = r - a * nb;
       double s = 0.0;
       if (use23)
-        for (int q = 0; q < n23; ++q) {
-          if (d23[q] < 0) continue;
-          const NbrEntry ef = A.nbr[it.fbase + f23[q]];
-          const int nf = A.nao[ef.other];
-          const double *c = A.C.data + A.C.offs[ef.cblk] + ((int64_t)(al0 + al) * na + a) * nf;
-          const double *d = A.D.data + A.D.offs[d23[q]] + b;
-          double t = 0.0;
-          for (int f = 0; f < nf; ++f) t = fma(c[f], d[f * nb], t);
-          s = fma((double)w23[q], t, s);
-        }
+#pragma unroll 4
+        for (int q = 0; q < n23; ++q)
+          if (d23[q] >= 0)
+            s = fma((double)w23[q], Q[((int64_t)f23[q] * pA + al0) * per2 + idx], s);
       Z2[idx] = s;
     }
     __syncthreads();
@@ -120,32 +171,78 @@ __global__ void __launch_bounds__(kThreads) k_adj_r(ContractArgs A) {
   if (threadIdx.x == 0) atomicAdd(A.macs + 0, macs);
 }
 
-// dV_AB[al][be] = -1/2 sum over active G of sum_{b,g} C_BG[be][b][g] R[al][b][(G,g)].
-__global__ void __launch_bounds__(kThreads) k_adj_dv(ContractArgs A) {
-  const int64_t w = A.w0 + blockIdx.x;
-  if (w >= A.w1) return;
+// dV_AB[al][be] = -1/2 sum over active G of sum_{b,g} C_BG[be][b][g] R[al][b][(G,g)],
+// one block per 32 al x 64 be of a pair: the product over (b, g) from shared
+// chunks of DV_K, 2 x 4 outputs a thread (six shared loads for eight
+// multiply-adds).  One block per pair with one output a thread read both
+// operands from global memory per multiply-add: 8.2 ms for what the FP64 units
+// do in 4.
+constexpr int DV_AL = 32, DV_BE = 64, DV_K = 32;
+__global__ void __launch_bounds__(kThreads) k_adj_dv(ContractArgs A, int nta, int ntb) {
+  __shared__ double Rs[DV_AL][DV_K + 1], Cs[DV_BE][DV_K + 1];
+  const int64_t w = A.w0 + blockIdx.x / (nta * ntb);
   const WorkItem it = A.items[w];
+  if (A.sym && it.role == 2) return;  // written by its mirror
+  const int tile = blockIdx.x % (nta * ntb);
   const int pA = A.nabf[it.a], pB = A.nabf[it.b], nb = A.nao[it.b];
+  const int al0 = tile / ntb * DV_AL, be0 = tile % ntb * DV_BE;
+  if (al0 >= pA || be0 >= pB) return;
   const int ncol = A.ncol[it.b];
   const double *R = A.scratch + A.p_off[w - A.w0];
-  double *out = A.dv + A.V.offs[it.vblk];
-  for (int o = threadIdx.x; o < pA * pB; o += kThreads) {
-    const int al = o / pB, be = o - al * pB;
-    double s = 0.0;
-    for (int g_ = 0; g_ < it.nG; ++g_) {
-      if (!(A.wg_flags[it.wg_off + g_] & 0xFu)) continue;
-      const NbrEntry eg = A.nbr[it.gbase + g_];
-      const int ng = A.nao[eg.other];
-      const double *c = A.C.data + A.C.offs[eg.cblk] + (int64_t)be * nb * ng;
-      const double *r = R + (int64_t)al * nb * ncol + eg.aopre;
-      for (int b = 0; b < nb; ++b)
-        for (int g = 0; g < ng; ++g) s = fma(c[b * ng + g], r[(int64_t)b * ncol + g], s);
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  double s[2][4] = {{0.0, 0.0, 0.0, 0.0}, {0.0, 0.0, 0.0, 0.0}};
+  for (int g_ = 0; g_ < it.nG; ++g_) {
+    if (!(A.wg_flags[it.wg_off + g_] & 0xFu)) continue;
+    const NbrEntry eg = A.nbr[it.gbase + g_];
+    const int ng = A.nao[eg.other], n = nb * ng;
+    const double *C = A.C.data + A.C.offs[eg.cblk];
+    for (int k0 = 0; k0 < n; k0 += DV_K) {
+      const int kk = threadIdx.x & 31, k = k0 + kk, b = k / ng, g = k - b * ng;
+      __syncthreads();
+      for (int r = threadIdx.x >> 5; r < DV_AL; r += kThreads / 32)
+        Rs[r][kk] = k < n && al0 + r < pA
+                        ? R[((int64_t)(al0 + r) * nb + b) * ncol + eg.aopre + g] : 0.0;
+      for (int r = threadIdx.x >> 5; r < DV_BE; r += kThreads / 32)
+        Cs[r][kk] = k < n && be0 + r < pB ? C[(int64_t)(be0 + r) * n + k] : 0.0;
+      __syncthreads();
+      const int m = min(DV_K, n - k0);
+      for (int q = 0; q < m; ++q) {
+        const double x0 = Rs[ty][q], x1 = Rs[ty + 16][q];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const double c = Cs[tx + 16 * j][q];
+          s[0][j] = fma(c, x0, s[0][j]);
+          s[1][j] = fma(c, x1, s[1][j]);
+        }
+      }
     }
-    out[(int64_t)al * pB + be] = -0.5 * s;
   }
+  // the mirror pair's V block, found among the work items (the V blocks in key order)
+  double *mir = nullptr;
+  if (A.sym && it.role == 1) {
+    const uint64_t key = hk_pack(it.b, it.a, -it.n[0], -it.n[1], -it.n[2]);
+    int64_t lo = 0, hi = A.nitems - 1;
+    while (lo < hi) {
+      const int64_t mid = (lo + hi) >> 1;
+      const WorkItem &m = A.items[mid];
+      if (hk_pack(m.a, m.b, m.n[0], m.n[1], m.n[2]) < key) lo = mid + 1; else hi = mid;
+    }
+    mir = A.dv + A.V.offs[A.items[lo].vblk];
+  }
+  double *out = A.dv + A.V.offs[it.vblk];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int al = al0 + ty + 16 * i, be = be0 + tx + 16 * j;
+      if (al >= pA || be >= pB) continue;
+      out[(int64_t)al * pB + be] = -0.5 * s[i][j];
+      if (mir) mir[(int64_t)be * pA + al] = -0.5 * s[i][j];
+    }
 }
 
-// dC_BG[be][b][g] += -1/2 sum_al V_AB[al][be] R[al][b][(G,g)]   (C in the B role)
+// dC_BG[be][b][g] += -1/2 sum_al V_AB[al][be] R[al][b][(G,g)]   (C in the B
+// role; twice that where it stands for the mirror's A role too)
 __global__ void __launch_bounds__(kThreads) k_adj_dcb(ContractArgs A) {
   const PairLoc L = locate(A, blockIdx.x, true);
   const WorkItem it = A.items[L.w];
@@ -156,12 +253,13 @@ __global__ void __launch_bounds__(kThreads) k_adj_dcb(ContractArgs A) {
   const double *V = A.V.data + A.V.offs[it.vblk];
   const double *R = A.scratch + A.p_off[L.w - A.w0] + eg.aopre;
   unsigned long long *acc = A.dcacc + 2 * A.C.offs[eg.cblk];
+  const double half = A.sym ? -1.0 : -0.5;
   for (int o = threadIdx.x; o < pB * nb * ng; o += kThreads) {
     const int be = o / (nb * ng), r = o - be * nb * ng, b = r / ng, g = r - b * ng;
     double s = 0.0;
     for (int al = 0; al < pA; ++al)
       s = fma(V[(int64_t)al * pB + be], R[((int64_t)al * nb + b) * ncol + g], s);
-    fx_add(acc + 2 * o, -0.5 * s, A.err);
+    fx_add(acc + 2 * o, half * s, A.err);
   }
 }
 
@@ -204,6 +302,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_dca(ContractArgs A) {
   const double *Dab = use14 ? A.D.data + A.D.offs[it.dab] : nullptr;
   const double *Dfb = use23 ? A.D.data + A.D.offs[dFB] : nullptr;
   const double *Ybase = A.scratch + A.y_off[L.w - A.w0];
+  const double *T3 = A.scratch + A.t3_off[L.w - A.w0];
   unsigned long long *acc = A.dcacc + 2 * A.C.offs[ef.cblk];
   const int per1 = nb * nf, per2 = na * nb;
   const int ach = max(1, min(pA, (kChunk / 2) / max(per1, per2)));
@@ -229,19 +328,12 @@ __global__ void __launch_bounds__(kThreads) k_adj_dca(ContractArgs A) {
     }
     // Ts[al][a][b] = sum_G w23 sum_g D_AG[a][g] Y[al][b][(G,g)]
     for (int idx = threadIdx.x; idx < ac * per2; idx += kThreads) {
-      const int al = idx / per2, r = idx - al * per2, a = r / nb, b = r - a * nb;
       double s = 0.0;
       if (use23)
-        for (int q = 0; q < n23; ++q) {
-          if (d23[q] < 0) continue;
-          const NbrEntry eg = A.nbr[it.gbase + g23[q]];
-          const int ng = A.nao[eg.other];
-          const double *y = Ybase + ((int64_t)(al0 + al) * nb + b) * ncol + eg.aopre;
-          const double *d = A.D.data + A.D.offs[d23[q]] + a * ng;
-          double t = 0.0;
-          for (int g = 0; g < ng; ++g) t = fma(d[g], y[g], t);
-          s = fma((double)w23[q], t, s);
-        }
+#pragma unroll 4
+        for (int q = 0; q < n23; ++q)
+          if (d23[q] >= 0)
+            s = fma((double)w23[q], T3[((int64_t)g23[q] * pA + al0) * per2 + idx], s);
       Ts[idx] = s;
     }
     __syncthreads();
@@ -267,13 +359,20 @@ __global__ void k_fx_to_double_adj(const unsigned long long *acc, int64_t n, dou
 
 }  // namespace
 
-cudaError_t launch_adjoint(const ContractArgs &a, cudaStream_t st) {
+cudaError_t launch_adjoint(const ContractArgs &a, int maxabf, cudaStream_t st) {
+  if (a.nwf > 0) k_adj_q<<<(unsigned)a.nwf, kThreads, 0, st>>>(a);
   if (a.nwg > 0) {
     k_adj_r<<<(unsigned)a.nwg, kThreads, 0, st>>>(a);
     k_adj_dcb<<<(unsigned)a.nwg, kThreads, 0, st>>>(a);
   }
-  if (a.w1 > a.w0) k_adj_dv<<<(unsigned)(a.w1 - a.w0), kThreads, 0, st>>>(a);
-  if (a.nwf > 0) k_adj_dca<<<(unsigned)a.nwf, kThreads, 0, st>>>(a);
+  if (a.w1 > a.w0) {
+    const int nta = (maxabf + DV_AL - 1) / DV_AL, ntb = (maxabf + DV_BE - 1) / DV_BE;
+    k_adj_dv<<<(unsigned)((a.w1 - a.w0) * nta * ntb), kThreads, 0, st>>>(a, nta, ntb);
+  }
+  if (!a.sym) {
+    if (a.nwg > 0) k_adj_t3<<<(unsigned)a.nwg, kThreads, 0, st>>>(a);
+    if (a.nwf > 0) k_adj_dca<<<(unsigned)a.nwf, kThreads, 0, st>>>(a);
+  }
   return cudaGetLastError();
 }
 

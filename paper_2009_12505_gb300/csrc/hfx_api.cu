@@ -1902,31 +1902,41 @@ hfx_status hfx_grad(hfx_ctx *ctx, double *dC, double *dV) {
   CK(cudaMemsetAsync(dvout.p, 0, sizeof(double) * (nV ? nV : 1), st));
   CK(cudaMemsetAsync(ctx->d_err.p, 0, sizeof(unsigned), st));
   CK(cudaMemsetAsync(ctx->d_counters.p + 8, 0, sizeof(unsigned long long) * 7, st));
-  // waves over the pairs: Y and R per pair
+  // waves over the pairs: R and Q per pair, and Y and T3 unless the B role
+  // stands for the A role too (Hermitian V and D)
+  const bool sym = ctx->sym;
+  const int maxabf = *std::max_element(ctx->nabf.begin(), ctx->nabf.end());
   const size_t budget = scratch_budget_doubles();
   const size_t nit = ctx->items.size();
   size_t w0 = 0;
   while (w0 < nit) {
     size_t w1 = w0, used = 0;
-    std::vector<int64_t> yo, ro;
+    std::vector<int64_t> ro, qo, yo, to;
     while (w1 < nit) {
       const WorkItem &it = ctx->items[w1];
       const int64_t ysz = (int64_t)ctx->nabf[it.a] * ctx->nao[it.b] * ctx->aotot[it.b];
-      if (w1 > w0 && used + 2 * ysz > budget) break;
-      yo.push_back((int64_t)used);
-      ro.push_back((int64_t)used + ysz);
-      used += 2 * ysz;
+      const int64_t per = (int64_t)ctx->nabf[it.a] * ctx->nao[it.a] * ctx->nao[it.b];
+      const int64_t qsz = it.nF * per, tsz = sym ? 0 : it.nG * per, y = sym ? 0 : ysz;
+      if (w1 > w0 && used + ysz + qsz + y + tsz > budget) break;
+      ro.push_back((int64_t)used);
+      qo.push_back((int64_t)used + ysz);
+      yo.push_back((int64_t)used + ysz + qsz);
+      to.push_back((int64_t)used + ysz + qsz + y);
+      used += ysz + qsz + y + tsz;
       ++w1;
     }
     const size_t nw = w1 - w0;
     std::vector<int64_t> offs(yo);
     offs.insert(offs.end(), ro.begin(), ro.end());
+    offs.insert(offs.end(), to.begin(), to.end());
+    offs.insert(offs.end(), qo.begin(), qo.end());
     CK(ctx->d_scratch.reserve(std::max<size_t>(used, 1)));
     CK(ctx->d_waveoffs.reserve(offs.size()));
     CK(cudaMemcpyAsync(ctx->d_waveoffs.p, offs.data(), sizeof(int64_t) * offs.size(),
                        cudaMemcpyHostToDevice, st));
     ContractArgs c{};
     c.items = ctx->d_items.p;
+    c.nitems = (int64_t)nit;
     c.w0 = (int64_t)w0;
     c.w1 = (int64_t)w1;
     c.wg_base = ctx->items[w0].wg_off;
@@ -1948,17 +1958,18 @@ hfx_status hfx_grad(hfx_ctx *ctx, double *dC, double *dV) {
     c.scratch = ctx->d_scratch.p;
     c.y_off = ctx->d_waveoffs.p;
     c.p_off = ctx->d_waveoffs.p + nw;
-    c.t3_off = c.q_off = c.y_off;
+    c.t3_off = ctx->d_waveoffs.p + 2 * nw;
+    c.q_off = ctx->d_waveoffs.p + 3 * nw;
     c.acc = ctx->d_acc.p;
     c.macs = ctx->d_counters.p + 8;
     c.err = ctx->d_err.p;
-    c.sym = 0;
-    c.skip = 2u | 4u | 8u | 16u | 32u | 64u;  // Y only
+    c.sym = sym ? 1 : 0;
+    c.skip = (sym ? 1u : 0u) | 2u | 4u | 8u | 16u | 32u | 64u;  // Y only, if at all
     c.dcacc = dcacc.p;
     c.dv = dvout.p;
     int nl = 0;
     CK(launch_contract_fp64(c, st, nullptr, &nl));
-    CK(launch_adjoint(c, st));
+    CK(launch_adjoint(c, maxabf, st));
     CK(cudaStreamSynchronize(st));
     w0 = w1;
   }

@@ -151,6 +151,7 @@ struct ScreenArgs {
 // Arguments of the contraction kernels for one wave of work items [w0, w1).
 struct ContractArgs {
   const WorkItem *items;
+  int64_t nitems;            // all work items (the adjoint finds mirrors among them)
   int64_t w0, w1;
   int64_t wg_base, wf_base;  // items[w0].wg_off, items[w0].wf_off
   int64_t nwg, nwf;          // (w,g) and (w,f) pairs in the wave
@@ -191,8 +192,9 @@ cudaError_t launch_collect_keys(const unsigned long long *keys, uint64_t cap,
 // Launches the seven FP64 contraction kernels; ev (8 events or null) is recorded
 // before the first and after each kernel.  Returns the number of launches in *nl.
 cudaError_t launch_contract_fp64(const ContractArgs &a, cudaStream_t st, cudaEvent_t *ev, int *nl);
-// Adjoint kernels for one wave (Y in y_off, R in p_off).
-cudaError_t launch_adjoint(const ContractArgs &a, cudaStream_t st);
+// Adjoint kernels for one wave (R in p_off, Q in q_off; without A.sym also Y in
+// y_off and T3 in t3_off); maxabf: the most ABFs of an atom.
+cudaError_t launch_adjoint(const ContractArgs &a, int maxabf, cudaStream_t st);
 cudaError_t launch_fx_to_double(const unsigned long long *acc, int64_t n, double *out,
                                 cudaStream_t st);
 // E_X = 1/2 the sum of n per-block partials, in the fixed order of the build.
