@@ -161,12 +161,12 @@ struct hfx_ctx {
   int split_ks = 0;
   DevBuf<__nv_bfloat16> d_cy, d_c4, d_vs, d_ps, d_cz;
   DevBuf<int16_t> d_cy_e, d_c4_e, d_vs_e, d_ps_e, d_cz_e;
-  DevBuf<int64_t> d_cz_meta;      // cz_base, cz_rowpre
+  DevBuf<int64_t> d_cz_meta;      // cz_base, cz_rowpre, czw_base, czw_rowpre
   DevBuf<int32_t> d_kofs, d_ktotZ;
   DevBuf<int16_t> d_colG;          // per (atom, column): index of its neighbour entry
   DevBuf<int64_t> d_coloff;        // per atom: first column in d_colG
   std::vector<int32_t> ktotZ_h;  // per atom: sum of 16 ceil(nao / 16) over its neighbours
-  int64_t h_cz_rows = 0;
+  int64_t h_cz_rows = 0, h_czw_rows = 0;
   // D digit tiles for the D_FG / D_FB products
   DevBuf<__nv_bfloat16> d_dz, d_dzero;
   DevBuf<int64_t> d_dz_off;
@@ -174,8 +174,7 @@ struct hfx_ctx {
   DevBuf<unsigned long long> d_de;
   int64_t dz_nd = -1;           // D blocks the tile metadata was built for (-1: stale)
   int dz_ks = 0;
-  int kbmax = 16;
-  ZcPlanShape zc_shape{16, 16, 0};
+  ZcPlanShape zc_shape{};
   int nsm = 0;
   DevBuf<ZcJob> d_zcjobs;
   DevBuf<ZcEnt> d_zcents;
@@ -578,7 +577,10 @@ hfx_status split_prepare(hfx_ctx *ctx, int ks) {
     vs_base[e + 1] = vs_base[e] + ntv * ctx->ktY[it.b] * ks * NT * TK;
   }
   // C as rows (al, a), K = F blocks of width 16 or 32
-  std::vector<int64_t> cz_base(n + 1, 0), cz_row(n + 1, 0);
+  // (once for k_zc, atoms of at most 16 AOs; when the cell has larger atoms, all
+  // of them once more in k_zcw's rows)
+  std::vector<int64_t> cz_base(n + 1, 0), cz_row(n + 1, 0), czw_base(n + 1, 0), czw_row(n + 1, 0);
+  const bool wide = *std::max_element(ctx->nao.begin(), ctx->nao.end()) > 16;
   std::vector<int32_t> kofs(ctx->nbr.size()), ktotZ(n);
   for (int x = 0; x < n; ++x) {
     int32_t k = 0;
@@ -587,15 +589,27 @@ hfx_status split_prepare(hfx_ctx *ctx, int ks) {
       k += ctx->nao[ctx->nbr[q].other] <= 16 ? 16 : 32;
     }
     ktotZ[x] = k;
-    const int64_t mtz = ((int64_t)ctx->nabf[x] * ctx->nao[x] + TM - 1) / TM;
+    const int64_t mtz =
+        ctx->nao[x] <= 16 ? ((int64_t)ctx->nabf[x] * ctx->nao[x] + TM - 1) / TM : 0;
+    const int64_t mtw = wide ? zc_tiles(ctx->nabf[x], ctx->nao[x]) : 0;
     cz_row[x + 1] = cz_row[x] + mtz * TM;
     cz_base[x + 1] = cz_base[x] + mtz * (int64_t)k * ks * TM;
+    czw_row[x + 1] = czw_row[x] + mtw * TM;
+    czw_base[x + 1] = czw_base[x] + mtw * (int64_t)k * ks * TM;
   }
   ctx->h_cz_rows = cz_row[n];
-  CK(ctx->d_cz.reserve(cz_base[n]));
-  CK(ctx->d_cz_e.reserve(cz_row[n]));
+  ctx->h_czw_rows = czw_row[n];
+  // k_zcw's rows follow k_zc's
+  for (int x = 0; x <= n; ++x) {
+    czw_row[x] += cz_row[n];
+    czw_base[x] += cz_base[n];
+  }
+  CK(ctx->d_cz.reserve(czw_base[n]));
+  CK(ctx->d_cz_e.reserve(czw_row[n]));
   std::vector<int64_t> czm(cz_base);
   czm.insert(czm.end(), cz_row.begin(), cz_row.end());
+  czm.insert(czm.end(), czw_base.begin(), czw_base.end());
+  czm.insert(czm.end(), czw_row.begin(), czw_row.end());
   CK(ctx->d_cz_meta.reserve(czm.size()));
   CK(cudaMemcpyAsync(ctx->d_cz_meta.p, czm.data(), sizeof(int64_t) * czm.size(),
                      cudaMemcpyHostToDevice, st));
@@ -674,24 +688,14 @@ hfx_status dz_prepare_meta(hfx_ctx *ctx, int ks) {
     off[e + 1] = off[e] + (int64_t)ks * R * kb;
   }
   std::vector<int32_t> aoff(n + 1, 0);
-  int kbmax = 16, naomax = 1, naomin = 1 << 30;
+  uint64_t present = 0;
   for (int x = 0; x < n; ++x) {
     aoff[x + 1] = aoff[x] + ctx->nao[x];
-    if (ctx->nao[x] > 16) kbmax = 32;
     if (ctx->nao[x] > 32)
       return fail(ctx, HFX_E_ARG, "the split modes support at most 32 NAOs per atom");
-    naomax = std::max(naomax, ctx->nao[x]);
-    naomin = std::min(naomin, ctx->nao[x]);
+    present |= 1ull << ctx->nao[x];
   }
-  // staged Y rows per tile: al rows spanned by 128 (al, a) rows, all b (plus
-  // 2 pairs of padding per al), the 16-column blocks of one G; for the small
-  // class (jobs whose blocks have at most 16 AOs) with the largest such atom
-  int naosmall = 1;
-  for (int x = 0; x < n; ++x)
-    if (ctx->nao[x] <= 16) naosmall = std::max(naosmall, ctx->nao[x]);
-  ctx->zc_shape = ZcPlanShape{kbmax, naomax,
-                              (127 / naomin + 2) * (naomax * 16 + 2) * 8 * ((naomax + 15) / 16),
-                              (127 / naomin + 2) * (naosmall * 16 + 2) * 8};
+  ctx->zc_shape = split_zc_shape(present);
   CK(ctx->d_dz.reserve(std::max<int64_t>(off[nd], 1)));
   CK(ctx->d_dz_off.reserve(std::max<int64_t>(nd, 1)));
   CK(ctx->d_dij.reserve(std::max<int64_t>(2 * nd, 1)));
@@ -708,7 +712,6 @@ hfx_status dz_prepare_meta(hfx_ctx *ctx, int ks) {
   CK(cudaStreamSynchronize(st));
   ctx->dz_nd = nd;
   ctx->dz_ks = ks;
-  ctx->kbmax = kbmax;
   if (!ctx->nsm) {
     int dev = 0, sm = 0;
     CK(cudaGetDevice(&dev));
@@ -749,6 +752,7 @@ SplitShared split_shared(hfx_ctx *ctx) {
   S.acc = ctx->d_acc.p;
   S.err = ctx->d_err.p;
   S.sym = ctx->sym ? 1 : 0;
+  S.ks = ctx->dz_ks;
   S.cy = ctx->d_cy.p;
   S.cy_e = ctx->d_cy_e.p;
   S.c4 = ctx->d_c4.p;
@@ -762,12 +766,15 @@ SplitShared split_shared(hfx_ctx *ctx) {
   S.cz_e = ctx->d_cz_e.p;
   S.cz_base = ctx->d_cz_meta.p;
   S.cz_rowpre = ctx->d_cz_meta.p + (n + 1);
+  S.czw_base = ctx->d_cz_meta.p + 2 * (n + 1);
+  S.czw_rowpre = ctx->d_cz_meta.p + 3 * (n + 1);
   S.kofs = ctx->d_kofs.p;
   S.ktotZ = ctx->d_ktotZ.p;
   S.Dd = ctx->K[2].data.p;
   S.Do = ctx->K[2].d_offs.p;
   S.dhash = DevHash{ctx->d_dhkeys.p, ctx->d_dhvals.p, ctx->dmask};
   S.h_cz_rows = ctx->h_cz_rows;
+  S.h_czw_rows = ctx->h_czw_rows;
   S.dz = ctx->d_dz.p;
   S.dzero = ctx->d_dzero.p;
   S.dz_off = ctx->d_dz_off.p;
@@ -1205,7 +1212,7 @@ hfx_status hfx_build(hfx_ctx *ctx, double theta, hfx_prec prec, int32_t nslices,
       CK(split_slice_inputs(SS, nslices, st));
       CK(split_slice_cz(SS, nslices, st));
       ctx->launches += (SS.h_cy_rows > 0) + (SS.h_c4_rows > 0) + (SS.h_v_rows > 0) +
-                       (SS.h_cz_rows > 0);
+                       (SS.h_cz_rows > 0) + (SS.h_czw_rows > 0);
     }
     if (ctx->dz_nd < 0 || ctx->dz_ks != nslices) {
       hfx_status s = dz_prepare_meta(ctx, nslices);

@@ -13,6 +13,27 @@ struct Job {
   int32_t mt, nt, k0, nk;
 };
 
+// Rows of k_zcw's A operand (C of an atom of na AOs as rows (al, a)): a 128-row
+// tile is 128 / u units of u rows, a unit holds slots
+// whole al, row s na + a of it the AO a of its al s; the unit's other rows are
+// zero.  A tile holds q al.  Whole al keep a row's a the same in every tile
+// and let the epilogue sum over al in place.  u is the smallest that gives at
+// least 85 % of the al that 128 / na would: a smaller unit splits fewer al
+// over two 16-row fragments.
+struct ZcRows {
+  int u, slots, q;
+};
+__host__ __device__ inline ZcRows zc_rows_of(int na) {
+  int u = 16;
+  while (u < 128 && 100 * (128 / u) * (u / na) < 85 * (128 / na)) u *= 2;
+  return ZcRows{u, u / na, (128 / u) * (u / na)};
+}
+// Row tiles of an atom of pA ABFs and na AOs.
+__host__ __device__ inline int zc_tiles(int pA, int na) {
+  const int q = zc_rows_of(na).q;
+  return (pA + q - 1) / q;
+}
+
 // One job of the D_FG / D_FB product: up to two column blocks (G index in
 // N[B], piece 1 = D_FG or 2 = D_FB) of work item w, over the F entries
 // [ent, ent + nent) of the union of their survivors.
@@ -27,10 +48,11 @@ struct ZcJob {
   int64_t ent;
 };
 
-// One F of a job: its K offset and width in the A operand, and per column
-// block the element offset of the D digit tile (-1: screened out, zeros).
+// 16 K of one F of a job (an F of more than 16 AOs has two entries): its K
+// offset in the A operand, and per column block the element offset of the D
+// digit tile (-1: screened out, zeros).
 struct ZcEnt {
-  int32_t kofs, kb;
+  int32_t kofs;
   int64_t dz[2];
 };
 
@@ -50,6 +72,7 @@ struct SplitShared {
   unsigned long long *acc;
   unsigned *err;
   int32_t sym;
+  int32_t ks;                      // digits per operand (D tile strides)
   // C of each atom transposed for Y: rows (b, G, g), K = beta
   __nv_bfloat16 *cy;
   const int64_t *cy_base, *cy_rowpre;
@@ -64,7 +87,9 @@ struct SplitShared {
   int16_t *vs_e;
   // C of each atom as rows (alpha, a), K = F blocks of width kb(F) = 16 ceil(nao(F)/16)
   __nv_bfloat16 *cz;
-  const int64_t *cz_base, *cz_rowpre;
+  const int64_t *cz_base, *cz_rowpre;    // atoms of at most 16 AOs (others: no rows)
+  const int64_t *czw_base, *czw_rowpre;  // the same in k_zcw's rows (ZcRows); no rows unless
+                                         // some atom has more than 16 AOs
   int16_t *cz_e;
   const int32_t *kofs;             // per neighbour entry: K offset of its F block
   const int32_t *ktotZ;            // per atom: total K of its F blocks
@@ -83,7 +108,7 @@ struct SplitShared {
   int32_t pd_pairs;                // f32 pairs of k_pdig's dynamic shared memory
   const int16_t *colG;             // per (atom, column): local index of its neighbour entry
   const int64_t *coloff;           // per atom: first column in colG
-  int64_t h_cy_rows, h_c4_rows, h_v_rows, h_cz_rows;  // host copies of the row totals
+  int64_t h_cy_rows, h_c4_rows, h_v_rows, h_cz_rows, h_czw_rows;  // host copies of the row totals
 };
 
 // Per-wave data.
@@ -135,12 +160,17 @@ cudaError_t split_dz_prepare(const SplitShared &S, int ks, cudaStream_t st);
 // W.zc_keys must then hold each key's start offset, keys in descending order)
 // and W.zc_ents.
 cudaError_t split_zc_plan(const SplitShared &S, const SplitWave &W, int fill, cudaStream_t st);
-// Launch shape of the D_FG / D_FB products: widest F block (16 or 32),
-// largest block output count, shared bytes of one staged Y block.
+// Shared bytes of staged Y for the D_FG / D_FB products: one block's buffer of
+// k_zc (blocks and atom A of at most 16 AOs), one tile's of k_zcw.
 struct ZcPlanShape {
-  int kbmax, nout_max, ybytes;
-  int ybytes_small;  // staged Y bytes for jobs whose blocks have at most 16 AOs
+  int ybytes_small, ybytes_wide;
 };
+// The shape for a system whose atoms have n AOs for the set bits n of present.
+ZcPlanShape split_zc_shape(uint64_t present);
+int split_zcw_ybytes(uint64_t present);
+// k_zcw over the jobs [jbeg, jend) of the wave's list.
+cudaError_t split_zcw_run(const SplitShared &S, const SplitWave &W, int ks, int ybytes, int nsm,
+                          int jbeg, int jend, int cta0, cudaStream_t st);
 // D_FG / D_FB products of one wave (after phase 0: needs the Y pairs).
 cudaError_t split_zc_run(const SplitShared &S, const SplitWave &W, int ks, const ZcPlanShape &P,
                          int nsm, int nsmall, cudaStream_t st);

@@ -39,18 +39,21 @@
 // warps 0-7 read an accumulator (warp w: TMEM lanes 32 (w % 4).., columns
 // 16 (w / 4)..), turn Z into f32 pairs, contract with Y in packed (f32x2)
 // double-float arithmetic, reduce over al through shared memory in a fixed
-// order and add
-// each finished block to the fixed-point Sigma (and its mirror for Hermitian
-// inputs) once per job.  Every wait is bounded; on expiry the kernel records
-// HFX_DEV_ERR_TIMEOUT, drains its copies and MMAs, frees TMEM and returns.
-#include <cuda_bf16.h>
-
-#include "hfx_split.h"
-#include "split_common.cuh"
+// order and add each finished block to the fixed-point Sigma (and its mirror
+// for Hermitian inputs) once per job.  Every wait is bounded; on expiry the
+// kernel records HFX_DEV_ERR_TIMEOUT, drains its copies and MMAs, frees TMEM and
+// returns.
+//
+// k_zc takes the jobs whose blocks and atom A have at most 16 AOs, k_zcw
+// (hfx_zcw.cu) the others.  k_zcw's second tensor-core product was tried for
+// small blocks too: 31.7 ms with 8 epilogue warps and 34.3 ms with 16, against
+// 24.7 (8-atom cell).  There the operand stream (30 KB a stage, 24 B/clk per SM
+// from L2) and the MMAs' shared-memory reads already take 17 of the 19 thousand
+// cycles of a tile.
+#include "zc_common.cuh"
 
 namespace split {
 
-constexpr int ZC_COLS = 32;                      // Z columns per job
 constexpr int ZC_KMAX = 640;                     // K per job: exact f32 group sums
 
 // Epilogue geometry for EPI epilogue warps (8 or 16): 4 warps cover the 128
@@ -63,35 +66,45 @@ struct ZcGeo {
   static constexpr int THREADS = (EPI + 3) * 32;     // + A/B loader, MMA issuer, Y loader
   static constexpr int OWN = 2 * 32 * 32 / ET;       // owned outputs per epilogue thread
 };
-constexpr long long ZC_WAIT = 2000000000ll;      // cycles per bounded wait
 // Staged Y rows of one al are padded by ZC_YPAD pairs, so the rows of the
 // few al a warp touches fall in different shared-memory banks.
 constexpr int ZC_YPAD = 2;
 
 __host__ __device__ __forceinline__ int kb_of(int nao) { return nao <= 16 ? 16 : 32; }
 
-// element offset of (r, c) in an [R x kb] K-major core-matrix tile
-__device__ __forceinline__ int tile_off_kb(int r, int c, int kb) {
-  return ((r >> 3) * (kb >> 3) + (c >> 3)) * 64 + (r & 7) * 8 + (c & 7);
+// element offset of (r, c) in an [R x 16] K-major core-matrix tile
+__device__ __forceinline__ int tile_off16(int r, int c) {
+  return ((r >> 3) * 2 + (c >> 3)) * 64 + (r & 7) * 8 + (c & 7);
 }
 
 // ---------------------------------------------------------------- operands
 
 // C of atom x as rows (al, a), K = F blocks (one exponent per row).
+// wide: the rows of k_zcw's operand (ZcRows), else row al nao + a.
 template <int KS>
-__global__ void k_slice_cz(SplitShared S) {
-  const int64_t grow = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+__global__ void k_slice_cz(SplitShared S, int wide) {
+  const int64_t *rowpre = wide ? S.czw_rowpre : S.cz_rowpre;
+  const int64_t grow = rowpre[0] + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
-  if (grow >= S.cz_rowpre[S.natoms]) return;
+  if (grow >= rowpre[S.natoms]) return;
   int lo = 0, hi = S.natoms - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (S.cz_rowpre[mid] <= grow) lo = mid; else hi = mid - 1;
+    if (rowpre[mid] <= grow) lo = mid; else hi = mid - 1;
   }
   const int x = lo;
-  const int r = (int)(grow - S.cz_rowpre[x]);
+  const int r = (int)(grow - rowpre[x]);
   const int nx = S.nao[x], px = S.nabf[x];
-  const bool live = r < px * nx;
+  const int mt = r / 128, rr = r - mt * 128;
+  bool live = r < px * nx;
+  int64_t src = r;
+  if (wide) {
+    const ZcRows R = zc_rows_of(nx);
+    const int slot = (rr & (R.u - 1)) / nx;
+    const int al = mt * R.q + (rr / R.u) * R.slots + slot;
+    live = slot < R.slots && al < px;
+    src = live ? (int64_t)al * nx + (rr & (R.u - 1)) - slot * nx : 0;
+  }
   const int64_t base = S.nc_start[x];
   const int n = (int)(S.nc_start[x + 1] - base);
   const int ktot = S.ktotZ[x];
@@ -101,25 +114,25 @@ __global__ void k_slice_cz(SplitShared S) {
       const NbrEntry &e = S.nbr[base + q];
       const int nf = S.nao[e.other];
       for (int f = lane; f < nf; f += 32)
-        mbits = max(mbits, __double_as_longlong(S.Cd[S.Co[e.cblk] + (int64_t)r * nf + f]) &
+        mbits = max(mbits, __double_as_longlong(S.Cd[S.Co[e.cblk] + src * nf + f]) &
                                0x7FFFFFFFFFFFFFFFll);
     }
   for (int o = 16; o; o >>= 1) mbits = max(mbits, __shfl_xor_sync(0xffffffffu, mbits, o));
   const int ex = row_exponent(mbits);
   if (lane == 0) S.cz_e[grow] = (int16_t)max(-30000, ex);
-  const int mt = r / 128, rr = r - mt * 128;
-  __nv_bfloat16 *tile0 = S.cz + S.cz_base[x] + (int64_t)mt * ktot * KS * 128;
+  __nv_bfloat16 *tile0 = S.cz + (wide ? S.czw_base : S.cz_base)[x] + (int64_t)mt * ktot * KS * 128;
   for (int q = 0; q < n; ++q) {
     const NbrEntry &e = S.nbr[base + q];
     const int nf = S.nao[e.other], kb = kb_of(nf);
     __nv_bfloat16 *tile = tile0 + (int64_t)S.kofs[base + q] * KS * 128;
     for (int f = lane; f < kb; f += 32) {
-      const double v = (live && f < nf) ? S.Cd[S.Co[e.cblk] + (int64_t)r * nf + f] : 0.0;
+      const double v = (live && f < nf) ? S.Cd[S.Co[e.cblk] + src * nf + f] : 0.0;
       int d[KS];
       to_digits<KS>(v, ex, d);
 #pragma unroll
       for (int s = 0; s < KS; ++s)
-        tile[(int64_t)s * kb * 128 + tile_off_kb(rr, f, kb)] = __int2bfloat16_rn(d[s]);
+        tile[(int64_t)((f >> 4) * KS + s) * 16 * 128 + tile_off16(rr, f & 15)] =
+            __int2bfloat16_rn(d[s]);
     }
   }
 }
@@ -139,8 +152,8 @@ __global__ void k_dz_exp(SplitShared S) {
   }
 }
 
-// D block (i, j, n) as the transposed digit tile [digit][R x kb]: rows y of
-// atom j (R = 16 or 32), K = x of atom i (kb = 16 or 32), exponent per y.
+// D block (i, j, n) as transposed digit tiles [K half][digit][R x 16]: rows y
+// of atom j (R = 16 or 32), K = x of atom i (16 per half), exponent per y.
 template <int KS>
 __global__ void k_dz_slice(SplitShared S) {
   const int64_t e = blockIdx.x;
@@ -158,7 +171,7 @@ __global__ void k_dz_slice(SplitShared S) {
     to_digits<KS>(v, ex, d);
 #pragma unroll
     for (int s = 0; s < KS; ++s)
-      t[(int64_t)s * R * kb + tile_off_kb(y, x, kb)] = __int2bfloat16_rn(d[s]);
+      t[(int64_t)((x >> 4) * KS + s) * R * 16 + tile_off16(y, x & 15)] = __int2bfloat16_rn(d[s]);
   }
 }
 
@@ -170,32 +183,23 @@ __global__ void k_dz_slice(SplitShared S) {
 // start offsets, and the fill pass places each job in its key's range, so the
 // list runs longest first (longest-processing-time order).
 constexpr int ZC_NCOST = 256;
-constexpr int ZC_NKEYS = 2 * ZC_NCOST;
 __device__ __forceinline__ int zc_cost_key(int mtz, int k) {
   return min(ZC_NCOST - 1, (mtz * (k / 16) + 3) / 4);
 }
-// Size class of a job: small when atom A and every block it touches have at
-// most 16 AOs (outputs, Z columns and F entries), so its Y rows fit the
-// staging buffers of the fastest kernel variant and its job sums fit fewer
-// registers; small jobs take keys [0, 256), the others [256, 512), and the
-// host places the small class first, so each class is a contiguous,
-// longest-first range launched with its own variant.
+// Size class of a job: small when atom A, B and its Gs have at most 16 AOs
+// (outputs and Z columns): k_zc's; the others are k_zcw's.  F does not count: a
+// wide F block is two entries of 16 K.  Small jobs take keys [0, 256), the
+// others [256, 512), and the host places the small class first, so each class
+// is a contiguous, longest-first range with a launch of its own.
 __device__ __forceinline__ int zc_key(int mtz, int k, bool small) {
   return zc_cost_key(mtz, k) + (small ? 0 : ZC_NCOST);
-}
-
-// Job handed to CTA b in round r of the persistent loop: rounds alternate
-// direction (snake order), so over a longest-first list every CTA gets a
-// similar mix of long and short jobs.  The last round is partial.
-__device__ __forceinline__ int zc_job_of(int r, int b, int G) {
-  return r * G + ((r & 1) ? G - 1 - b : b);
 }
 
 // Runs of the union of a group's surviving F with at most ZC_KMAX K each: one
 // job per run.  Called by one lane per group.  fill == 0 only counts.
 __device__ void zc_plan_group(const SplitShared &S, const SplitWave &W, const WorkItem &it,
                               int32_t w, const int (&bg)[2], const int (&bp)[2], int nblk,
-                              int mtz, int fill, unsigned long long &macs,
+                              int fill, unsigned long long &macs,
                               unsigned long long &umacs) {
   const uint32_t *mr[2] = {nullptr, nullptr};
   for (int q = 0; q < nblk; ++q)
@@ -211,10 +215,11 @@ __device__ void zc_plan_group(const SplitShared &S, const SplitWave &W, const Wo
     ncv[q] = bp[q] == 1 ? S.nao[eg.other] : S.nao[it.b];
   }
   const unsigned long long rows = (unsigned long long)S.nabf[it.a] * S.nao[it.a];
-  // outputs and Z columns of both pieces are nao(B) and nao(G); the small
-  // class also bounds atom A (the outputs an epilogue thread owns)
+  // outputs and Z columns of both pieces are nao(B) and nao(G)
   bool small = S.nao[it.b] <= 16 && S.nao[it.a] <= 16;
   for (int q = 0; q < nblk; ++q) small = small && S.nao[(int)eg_n[q][0]] <= 16;
+  const int pA = S.nabf[it.a], na = S.nao[it.a];
+  const int mtz = small ? (pA * na + 127) / 128 : zc_tiles(pA, na);
   // cursor over the union bits: word wd, remaining bits u
   int wd = 0;
   uint32_t u = 0;
@@ -237,28 +242,28 @@ __device__ void zc_plan_group(const SplitShared &S, const SplitWave &W, const Wo
     const int wd0 = wd;
     const uint32_t u0 = u;
     const int f0 = f;
-    int n = 0, k = 0, kbm = 16;
+    int n = 0, k = 0;  // F and K of the run
     int fa = f;
     bool ma = true;
     while (ma) {
       const int kb = kb_of(S.nao[S.nbr[it.fbase + fa].other]);
       if (k + kb > ZC_KMAX) break;
       k += kb;
-      kbm = max(kbm, kb);
       ++n;
       ma = next(fa);
     }
     macs += (unsigned long long)mtz * 128 * ZC_COLS * k;
-    const int key = zc_key(mtz, k, small && kbm == 16);
+    const int key = zc_key(mtz, k, small);
+    const int nent = k / 16;
     int64_t eo = 0;
     if (!fill) {
       atomicAdd(W.njobs + 2, 1);
-      atomicAdd(W.njobs + 3, n);
+      atomicAdd(W.njobs + 3, nent);
       atomicAdd(W.zc_keys + key, 1);
     } else {
       atomicAdd(W.njobs + 2, 1);
       const int js = atomicAdd(W.zc_keys + key, 1);  // next slot of this key's range
-      eo = (int64_t)atomicAdd(W.njobs + 3, n);
+      eo = (int64_t)atomicAdd(W.njobs + 3, nent);
       ZcJob jb{};
       jb.w = w;
       jb.nblk = (int8_t)nblk;
@@ -266,18 +271,18 @@ __device__ void zc_plan_group(const SplitShared &S, const SplitWave &W, const Wo
         jb.g[q] = (int16_t)(q < nblk ? bg[q] : -1);
         jb.piece[q] = (int8_t)(q < nblk ? bp[q] : 0);
       }
-      jb.nent = n;
+      jb.nent = nent;
       jb.ent = eo;
       W.zc_jobs[js] = jb;
       // entries: rewind to the run start
       wd = wd0;
       u = u0;
       int fe = f0;
+      int64_t eq = eo;
       for (int q = 0; q < n; ++q) {
         const NbrEntry ef = S.nbr[it.fbase + fe];
         ZcEnt en{};
         en.kofs = S.kofs[it.fbase + fe];
-        en.kb = kb_of(S.nao[ef.other]);
         for (int c = 0; c < 2; ++c) {
           en.dz[c] = -1;
           if (c >= nblk || !((mr[c][fe >> 5] >> (fe & 31)) & 1u)) continue;
@@ -298,7 +303,13 @@ __device__ void zc_plan_group(const SplitShared &S, const SplitWave &W, const Wo
             umacs += rows * (unsigned long long)S.nao[ef.other] * ncv[c];
           }
         }
-        W.zc_ents[eo + q] = en;
+        W.zc_ents[eq++] = en;
+        if (S.nao[ef.other] > 16) {  // its second 16 K
+          en.kofs += 16;
+          for (int c = 0; c < 2; ++c)
+            if (en.dz[c] >= 0) en.dz[c] += (int64_t)S.ks * 16 * (ncv[c] <= 16 ? 16 : 32);
+          W.zc_ents[eq++] = en;
+        }
         if (q + 1 < n) next(fe);
       }
       // leave the cursor after the run
@@ -321,8 +332,7 @@ __global__ void __launch_bounds__(128) k_zc_plan(SplitShared S, SplitWave W, int
   const int wl = blockIdx.x * 4 + wib;
   if (wl >= W.nw) return;
   const WorkItem it = S.items[W.w0 + wl];
-  const int pA = S.nabf[it.a], na = S.nao[it.a], nb = S.nao[it.b];
-  const int mtz = (pA * na + 127) / 128;
+  const int nb = S.nao[it.b];
   unsigned long long macs = 0, umacs = 0;
   // lane 0 state: cursor (g, piece) and the open group
   int g = 0, piece = 1, nblk = 0, rows = 0, cg[2] = {0, 0}, cp[2] = {0, 0};
@@ -375,7 +385,7 @@ __global__ void __launch_bounds__(128) k_zc_plan(SplitShared S, SplitWave W, int
     if (lane < cnt) {
       const int *o = sgrp[wib][lane];
       const int bg[2] = {o[0], o[2]}, bp[2] = {o[1], o[3]};
-      zc_plan_group(S, W, it, (int32_t)(W.w0 + wl), bg, bp, o[4], mtz, fill, macs, umacs);
+      zc_plan_group(S, W, it, (int32_t)(W.w0 + wl), bg, bp, o[4], fill, macs, umacs);
     }
     __syncwarp();
     if (fin) break;
@@ -390,208 +400,14 @@ __global__ void __launch_bounds__(128) k_zc_plan(SplitShared S, SplitWave W, int
 
 // ---------------------------------------------------------------- product
 
-// Epilogue data of one job, written to shared memory by a few lanes when its
-// pair starts and read by every epilogue thread on each of the job's tiles.
-struct ZcEpiJob {
-  int64_t czrow0;    // first row of atom A's C exponents
-  int64_t y2off;     // the work item's Y pairs in the wave scratch
-  int64_t sg[2][2];  // block q: Sigma offset of its outputs, of their mirror (-1: none)
-  int pA, na, nb, mtz, nblk, R0b;
-  int nout[2], ncv[2], pc[2], gcb[2];
-};
-
 struct ZcSmem {
   uint64_t full[8], empty[8], tfull[2], tempty[2], yfull[2], yempty[2], drain;
   unsigned long long t_start;  // globaltimer at the start of the roles
   uint32_t tslot;
   int abort_f;
-  int stkb[8];  // K of the entry in each operand stage (16 or 32)
   int ecol[2][ZC_COLS];  // column exponents of the pair's jobs (column group q at q * CW)
   ZcEpiJob ej[2][2];     // [pair parity][job of the pair]
 };
-
-// Number of jobs CTA b receives from zc_job_of over a list of njobs.
-__device__ __forceinline__ int zc_cta_jobs(int njobs, int b, int G) {
-  const int full = njobs / G, rem = njobs - full * G;
-  return full + (((full & 1) ? G - 1 - b : b) < rem ? 1 : 0);
-}
-
-// Tile order of a CTA.  Its jobs r = 0 .. n - 1 run heaviest first (operand
-// stages x row tiles).  With PAIR, pair p is job n - 1 - p (light) and job p
-// (heavy), and their row tiles alternate while both have some: the MMAs of a
-// long tile then run beside the epilogue of a short one, where one job after
-// the other leaves the epilogue idle through the long tiles and the tensor
-// pipe idle through the short ones.  Without PAIR, pair p is job p alone.
-// Every role walks the same order.
-template <bool PAIR>
-struct ZcPair {
-  int r0, r1, m0, m1, t0, t1, last;
-  bool two;
-  __device__ __forceinline__ void begin(int p, int n) {
-    r0 = PAIR ? n - 1 - p : p;
-    r1 = PAIR ? p : -1;
-    two = PAIR && r1 < r0;
-    m0 = m1 = t0 = t1 = 0;
-    last = 1;
-  }
-  // next tile: job x of the pair (0: r0, 1: r1) and its row tile mt
-  __device__ __forceinline__ bool next(int &x, int &mt) {
-    const bool a = t0 < m0, b = t1 < m1;
-    if (!a && !b) return false;
-    x = (a && (!b || last == 1)) ? 0 : 1;
-    last = x;
-    mt = x ? t1++ : t0++;
-    return true;
-  }
-};
-
-template <class T>
-__device__ __forceinline__ void zc_swap(T &a, T &b) {
-  const T t = a;
-  a = b;
-  b = t;
-}
-
-__device__ __forceinline__ ZcJob zc_job(const SplitWave &W, int jbeg, int r) {
-  return W.zc_jobs[jbeg + zc_job_of(r, blockIdx.x, gridDim.x)];
-}
-
-// rows of a job's lone column block (16 or 32); two blocks have 16 each
-__device__ __forceinline__ int zc_rows(const SplitShared &S, const ZcJob &jb, const WorkItem &it) {
-  if (jb.nblk != 1) return 16;
-  const int ncb = jb.piece[0] == 1 ? S.nao[S.nbr[it.gbase + jb.g[0]].other] : S.nao[it.b];
-  return ncb <= 16 ? 16 : 32;
-}
-
-// block and first column cq of column group q of width CW: two 16-column
-// blocks take half the groups each; one block takes the groups below its R
-template <int CW>
-__device__ __forceinline__ int zc_group_block(int nblk, int R0b, int q, int &cq) {
-  const int jc = q * CW;
-  if (nblk == 2) { cq = jc & 15; return jc >> 4; }
-  cq = jc;
-  return jc < R0b ? 0 : -1;
-}
-
-// Epilogue data of job r, by one whole warp: lanes 0 .. 3 look up the Sigma
-// offsets of block lane / 2 (odd lanes: the mirror), lane 4 the scalars.  A
-// missing Sigma key fails the build, and the block is not added.
-__device__ __forceinline__ void zc_epi_job(const SplitShared &S, const SplitWave &W, int jbeg,
-                                           int r, int lane, ZcEpiJob &e) {
-  const ZcJob jb = zc_job(W, jbeg, r);
-  const WorkItem it = S.items[jb.w];
-  const int q = (lane >> 1) & 1, m = lane & 1;
-  int64_t t = -1;
-  bool miss = false;
-  if (lane < 4 && q < jb.nblk) {
-    const int pcb = q ? jb.piece[1] : jb.piece[0];
-    const bool mir = S.sym && (pcb == 2 || it.role == 1);
-    if (m == 0 || mir) {
-      if (pcb == 1) {
-        t = m == 0 ? dh_find(S.shash, hk_pack(it.a, it.b, it.n[0], it.n[1], it.n[2]))
-                   : dh_find(S.shash, hk_pack(it.b, it.a, -it.n[0], -it.n[1], -it.n[2]));
-      } else {
-        const NbrEntry eg = S.nbr[it.gbase + (q ? jb.g[1] : jb.g[0])];
-        const int n0 = it.n[0] + eg.n[0], n1 = it.n[1] + eg.n[1], n2 = it.n[2] + eg.n[2];
-        t = m == 0 ? dh_find(S.shash, hk_pack(it.a, eg.other, n0, n1, n2))
-                   : dh_find(S.shash, hk_pack(eg.other, it.a, -n0, -n1, -n2));
-      }
-      miss = t < 0;
-      if (miss) atomicOr(S.err, HFX_DEV_ERR_MISSING);
-    }
-  }
-  const bool bad = __shfl_sync(0xffffffffu, (int)miss, lane & ~1) |
-                   __shfl_sync(0xffffffffu, (int)miss, lane | 1);
-  if (lane < 4) e.sg[q][m] = bad ? -1 : t;
-  if (lane == 4) {
-    const int pA = S.nabf[it.a], na = S.nao[it.a], nb = S.nao[it.b];
-    e.czrow0 = S.cz_rowpre[it.a];
-    e.y2off = W.y2_off[(int)(jb.w - W.w0)];
-    e.pA = pA;
-    e.na = na;
-    e.nb = nb;
-    e.mtz = (pA * na + 127) / 128;
-    e.nblk = jb.nblk;
-    e.R0b = 16;
-#pragma unroll
-    for (int b = 0; b < 2; ++b) {
-      e.nout[b] = e.ncv[b] = e.pc[b] = e.gcb[b] = 0;
-      if (b < jb.nblk) {
-        const int ng = S.nao[S.nbr[it.gbase + jb.g[b]].other];
-        e.pc[b] = jb.piece[b];
-        e.gcb[b] = S.kofs[it.gbase + jb.g[b]] / 16;
-        e.ncv[b] = jb.piece[b] == 1 ? ng : nb;
-        e.nout[b] = jb.piece[b] == 1 ? nb : ng;
-      }
-    }
-    if (jb.nblk > 0) e.R0b = e.ncv[0] <= 16 ? 16 : 32;
-  }
-}
-
-// Column exponents of job r's column group hf (CW columns), by lanes < CW.
-template <int CW>
-__device__ __forceinline__ void zc_epi_ecol(const SplitShared &S, const SplitWave &W, int jbeg,
-                                            int r, int hf, int lane, int *ecol) {
-  if (lane >= CW) return;
-  const ZcJob jb = zc_job(W, jbeg, r);
-  const WorkItem it = S.items[jb.w];
-  int ncv0 = 0, R0b = 16;
-  if (jb.nblk > 0) {
-    ncv0 = jb.piece[0] == 1 ? S.nao[S.nbr[it.gbase + jb.g[0]].other] : S.nao[it.b];
-    R0b = ncv0 <= 16 ? 16 : 32;
-  }
-  int c0 = 0;
-  const int hb = zc_group_block<CW>(jb.nblk, R0b, hf, c0);
-  int e = -1000;
-  if (hb >= 0) {
-    const int pc = hb ? jb.piece[1] : jb.piece[0], g = hb ? jb.g[1] : jb.g[0];
-    const int at = pc == 1 ? S.nbr[it.gbase + g].other : it.b;
-    const int ncvh = S.nao[at];  // piece 1: nao(G); piece 2: nao(B)
-    const int cc = c0 + lane;
-    if (cc < ncvh) e = row_exponent((long long)S.de[S.aoff[at] + cc]);
-  }
-  ecol[hf * CW + lane] = e;
-}
-
-// Launch shape of k_zc: ybytes = shared bytes per staged Y block (0: the
-// epilogue reads Y from global memory), rs = outputs per block held in the
-// reduction buffer (16 or 32; the buffer is [column group][output][row]).
-struct ZcCfg {
-  int ybytes, rs;
-  int jbeg, jend;  // the launch's range of the job list
-  int cta0;        // first slot of its CTAs' busy times
-};
-
-// Y rows al in [al0, al0 + nal) of the 16-column block cb: [al][b][16] pairs.
-__device__ __forceinline__ const float2 *zc_y_global(const float2 *Y2, int cb, int pA, int nb,
-                                                     int al) {
-  return Y2 + (((int64_t)cb * pA + al) * nb) * 16;
-}
-
-// One operand stage's MMAs (K = KB): for each K step of 16 and block b, A
-// digit i times the block's B digits 0 .. KS - 1 - i stacked along N
-// (N = R (KS - i)) into TMEM columns b 16 KS + i R ..  Descriptors are the
-// stage's two base descriptors plus constant offsets (the 14-bit start field
-// cannot carry: shared addresses stay below 2^18).
-template <int KS, int KB>
-__device__ __forceinline__ void zc_stage_mmas(uint32_t a0, uint32_t b0, uint32_t dcol, int nblk,
-                                              int R, const uint32_t (&id16)[KS],
-                                              const uint32_t (&id32)[KS], bool first) {
-  constexpr uint32_t SBO = KB / 8 * 128;
-  const uint64_t adesc = umma::smem_desc(a0, 128, SBO);
-  const uint64_t bdesc = umma::smem_desc(b0, 128, SBO);
-#pragma unroll
-  for (int ks = 0; ks < KB / 16; ++ks)
-    for (int b = 0; b < nblk; ++b) {
-      const uint64_t bd = bdesc + (uint64_t)((b * (KS * 16 * KB * 2) + ks * 256) >> 4);
-#pragma unroll
-      for (int i = 0; i < KS; ++i) {
-        const uint64_t ad = adesc + (uint64_t)((i * (128 * KB * 2) + ks * 256) >> 4);
-        umma::mma_bf16(dcol + (uint32_t)(b * 16 * KS + i * R), ad, bd,
-                       R == 16 ? id16[i] : id32[i], (!first || ks || i) ? 1u : 0u);
-      }
-    }
-}
 
 // One row's contraction with Y in double-float: out[o] = sum_{c < cend} z[c]
 // yb[o so + c sc] for o < no, four outputs at a time; out[o] is stored at
@@ -690,30 +506,6 @@ __device__ __forceinline__ void zc_contract2(const uint64_t (&zh)[NP], const uin
   }
 }
 
-// Loader-warp view of a job: operand bases, its entries (lane l holds entry
-// held + l) and the B rows per block.
-struct ZcLd {
-  const __nv_bfloat16 *A;
-  int64_t ktot, ent;
-  int nent, nblk, Rl, mtz, held;
-  ZcEnt mine;
-};
-
-__device__ __forceinline__ void zc_ld_job(const SplitShared &S, const SplitWave &W, int jbeg,
-                                          int r, ZcLd &L) {
-  const ZcJob jb = zc_job(W, jbeg, r);
-  const WorkItem it = S.items[jb.w];
-  L.A = S.cz + S.cz_base[it.a];
-  L.ktot = S.ktotZ[it.a];
-  L.ent = jb.ent;
-  L.nent = jb.nent;
-  L.nblk = jb.nblk;
-  L.Rl = zc_rows(S, jb, it);
-  L.mtz = (S.nabf[it.a] * S.nao[it.a] + 127) / 128;
-  L.held = -1;
-  L.mine = ZcEnt{0, 0, {-1, -1}};
-}
-
 // Y-loader view of a job: its Y pairs, sizes and the 16-column blocks of Y
 // columns of each column block.
 struct ZcYJob {
@@ -742,24 +534,23 @@ __device__ __forceinline__ void zc_y_job(const SplitShared &S, const SplitWave &
   }
 }
 
-template <int KS, int KBM, int NST, int EPI, bool YST, bool PAIR>
+template <int KS, int NST, int EPI, bool YST, bool PAIR>
 __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
     k_zc(SplitShared S, SplitWave W, ZcCfg cfg) {
   constexpr int ZC_EPI = EPI, ZC_NQ = ZcGeo<EPI>::NQ, ZC_CW = ZcGeo<EPI>::CW,
                 ZC_ET = ZcGeo<EPI>::ET;
-  // owned outputs per epilogue thread, for the job sums of both paired jobs:
-  // na x (outputs of the job's blocks), at most 16 x 32 in the small class
-  // (atom A and blocks of at most 16 AOs), else 32 x 64 (two blocks of 16
-  // columns of piece 1 have nao(B) outputs each)
-  constexpr int ZC_OWN = PAIR && KBM == 16 ? (16 * 32 + ZC_ET - 1) / ZC_ET : ZcGeo<EPI>::OWN;
-  constexpr int A_BYTES = KS * 128 * KBM * 2;
-  constexpr int B_BYTES = KS * ZC_COLS * KBM * 2;
+  // owned outputs per epilogue thread, for the job sums of both paired jobs: na x
+  // (outputs of the job's blocks), at most 16 x 32
+  constexpr int ZC_OWN = (16 * 32 + ZC_ET - 1) / ZC_ET;
+  constexpr int ZC_RS = 16;  // outputs of a block in the reduction buffer
+  constexpr int A_BYTES = KS * 128 * 16 * 2;
+  constexpr int B_BYTES = KS * ZC_COLS * 16 * 2;
   constexpr int STG = A_BYTES + B_BYTES;
   constexpr int SH = 7 * (KS + 1);
   extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t *ybuf = smem + NST * STG;                                     // [2][2][ybytes]
-  float2 *red = reinterpret_cast<float2 *>(ybuf + 4 * cfg.ybytes);     // [ZC_NQ][rs][128]
-  ZcSmem *ctl = reinterpret_cast<ZcSmem *>(red + ZC_NQ * 128 * cfg.rs);
+  float2 *red = reinterpret_cast<float2 *>(ybuf + 4 * cfg.ybytes);     // [ZC_NQ][ZC_RS][128]
+  ZcSmem *ctl = reinterpret_cast<ZcSmem *>(red + ZC_NQ * 128 * ZC_RS);
   volatile int *abort_f = &ctl->abort_f;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -811,10 +602,10 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
       ZcPair<PAIR> pr;
       pr.begin(p, ncj);
       ZcLd L, Lo;  // L: the job of the current tile, Lo: the pair's other job
-      zc_ld_job(S, W, cfg.jbeg, pr.r0, L);
+      zc_ld_job<false>(S, W, cfg.jbeg, pr.r0, L);
       pr.m0 = L.mtz;
       if (pr.two) {
-        zc_ld_job(S, W, cfg.jbeg, pr.r1, Lo);
+        zc_ld_job<false>(S, W, cfg.jbeg, pr.r1, Lo);
         pr.m1 = Lo.mtz;
       }
       int cur = 0, x, mt;
@@ -833,7 +624,6 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
           const int nq = min(32, L.nent - q0);
           for (int qq = 0; qq < nq; ++qq, ++step) {
             const int kofs = __shfl_sync(0xffffffffu, L.mine.kofs, qq);
-            const int kb = __shfl_sync(0xffffffffu, L.mine.kb, qq);
             const long long d0 = __shfl_sync(0xffffffffu, (long long)L.mine.dz[0], qq);
             const long long d1 = __shfl_sync(0xffffffffu, (long long)L.mine.dz[1], qq);
             const int s = (int)(step % NST);
@@ -851,22 +641,18 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
               break;
             }
             uint8_t *st = smem + s * STG;
-            const uint32_t abytes = (uint32_t)(KS * 128 * kb * 2);
-            const uint32_t bbytes = (uint32_t)(KS * kb * 2) * (uint32_t)(L.nblk * L.Rl);
-            if (lane == 0) {
-              ctl->stkb[s] = kb;  // read by the MMA issuer after the stage lands
-              umma::mbar_arrive_expect_tx(&ctl->full[s], abytes + bbytes);
-            }
+            const uint32_t bbytes = (uint32_t)(KS * 16 * 2) * (uint32_t)(L.nblk * L.Rl);
+            if (lane == 0) umma::mbar_arrive_expect_tx(&ctl->full[s], A_BYTES + bbytes);
             __syncwarp();
             if (lane == 0) {
-              umma::bulk_g2s(st, L.A + ((int64_t)mt * L.ktot + kofs) * KS * 128, abytes,
+              umma::bulk_g2s(st, L.A + ((int64_t)mt * L.ktot + kofs) * KS * 128, A_BYTES,
                              &ctl->full[s]);
             } else if (has_b) {
-              // B stage block-major: block b's KS digits of Rl rows x kb at b KS 16 kb
+              // B stage block-major: block b's KS digits of Rl rows x 16 K at b KS 16 16
               const int64_t dz = cb == 0 ? d0 : d1;
               const __nv_bfloat16 *src = dz >= 0 ? S.dz + dz : S.dzero;
-              umma::bulk_g2s(st + A_BYTES + cb * (KS * 16 * kb * 2), src,
-                             (uint32_t)(KS * L.Rl * kb * 2), &ctl->full[s]);
+              umma::bulk_g2s(st + A_BYTES + cb * (KS * 16 * 16 * 2), src,
+                             (uint32_t)(KS * L.Rl * 16 * 2), &ctl->full[s]);
             }
           }
         }
@@ -985,10 +771,7 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
             }
             umma::fence_after_sync();
             const uint32_t a0 = sbase + (uint32_t)(s * STG);
-            if (KBM == 16 || ctl->stkb[s] == 16)
-              zc_stage_mmas<KS, 16>(a0, a0 + A_BYTES, dcol, nblk, R, idesc16, idesc32, q == 0);
-            else
-              zc_stage_mmas<KS, 32>(a0, a0 + A_BYTES, dcol, nblk, R, idesc16, idesc32, q == 0);
+            zc_stage_mmas<KS>(a0, a0 + A_BYTES, dcol, nblk, R, idesc16, idesc32, q == 0);
             umma::mma_commit(&ctl->empty[s]);
           }
           if (!ok) break;
@@ -1005,7 +788,7 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
     const int q4 = warp & 3, hf = warp >> 2;  // TMEM lane quarter, column group
     const int row = q4 * 32 + lane;
     const int et = threadIdx.x;  // 0 .. ZC_ET - 1
-    const int rs = cfg.rs;
+    constexpr int rs = ZC_RS;
     long long hand = 0;
     bool aborted = false;
     for (int p = 0; p < npair && !aborted; ++p) {
@@ -1018,7 +801,7 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
       // behind its tile barriers, and its data sit in the other parity.
       if (q4 < 2) {
         if (hf == 0 && (q4 == 0 || pr.two))
-          zc_epi_job(S, W, cfg.jbeg, q4 ? pr.r1 : pr.r0, lane, ctl->ej[pp][q4]);
+          zc_epi_job<false>(S, W, cfg.jbeg, q4 ? pr.r1 : pr.r0, lane, ctl->ej[pp][q4]);
       } else if (q4 == 2 || pr.two) {
         zc_epi_ecol<ZC_CW>(S, W, cfg.jbeg, q4 == 3 ? pr.r1 : pr.r0, hf, lane, ctl->ecol[q4 - 2]);
       }
@@ -1089,10 +872,7 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
 #pragma unroll
             for (int u = 0; u < 3; ++u)
               if (g0 + u < KS) {
-                if constexpr (ZC_CW == 8)
-                  umma::tmem_ld8_nowait(ta + (uint32_t)((g0 + u) * Rh), r[u]);
-                else
-                  umma::tmem_ld16_nowait(ta + (uint32_t)((g0 + u) * Rh), r[u]);
+                umma::tmem_ld16_nowait(ta + (uint32_t)((g0 + u) * Rh), r[u]);
               }
             umma::tmem_wait_ld();
 #pragma unroll
@@ -1124,7 +904,7 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
         // quarter's warps stage Z in rows 32 .. 63 of the reduction buffer
         // (unused by such a tile) and all epilogue warps share the contraction
         const int rv = min(128, pA * na - mt * 128);
-        if (PAIR && YST && KBM == 16 && rv <= 32) {
+        if (PAIR && YST && rv <= 32) {
           constexpr int NPT = ZC_CW / 2;
           if (q4 == 0 && hb >= 0 && rvalid) {
             float2 *zs = red + (int64_t)hf * rs * 128 + 32 + row;
@@ -1293,63 +1073,57 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
   }
 }
 
-// Y staged in shared memory (two buffers per block) with a shorter operand
-// ring, or read from global memory with a deeper ring.
-constexpr bool ZC_STAGE_Y = true;
-
+// Jobs are taken in heavy/light pairs by the four-stage variant; its fallbacks,
+// for cells whose staged Y does not fit next to four stages (three stages, then
+// Y read from global memory), keep one job at a time.  8 epilogue warps (2
+// column groups of 16): 16 warps (4 groups of 8) leave room for only two
+// operand stages next to the staged Y and were slower.
 template <int KS>
-cudaError_t zc_range_t(const SplitShared &S, const SplitWave &W, const ZcPlanShape &P, int nsm,
-                       int jbeg, int jend, int cta0, bool small, cudaStream_t st) {
+cudaError_t zc_range_t(const SplitShared &S, const SplitWave &W, int ybytes, int nsm, int jbeg,
+                       int jend, int cta0, cudaStream_t st) {
   const int blocks = (int)std::min<int64_t>(jend - jbeg, nsm);
   if (blocks <= 0) return cudaSuccess;
   constexpr size_t kMax = 227 * 1024;
-  const int rs = P.nout_max <= 16 ? 16 : 32;
-  auto smem_of = [&](int nst, int kbm, int ybytes, int nq) {
-    return (size_t)nst * KS * (128 + ZC_COLS) * kbm * 2 + 4 * (size_t)ybytes +
-           (size_t)nq * 128 * rs * sizeof(float2) + sizeof(ZcSmem) + 64;
+  auto smem_of = [&](int nst, int yb) {
+    return (size_t)nst * KS * (128 + ZC_COLS) * 16 * 2 + 4 * (size_t)yb +
+           (size_t)2 * 128 * 16 * sizeof(float2) + sizeof(ZcSmem) + 64;
   };
-  auto launch = [&](auto kern, int threads, int nst, int kbm, int ybytes, int nq) -> cudaError_t {
-    const size_t smem = smem_of(nst, kbm, ybytes, nq);
+  auto launch = [&](auto kern, int nst, int yb) -> cudaError_t {
+    const size_t smem = smem_of(nst, yb);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<blocks, threads, smem, st>>>(S, W, ZcCfg{ybytes, rs, jbeg, jend, cta0});
+    kern<<<blocks, ZcGeo<8>::THREADS, smem, st>>>(S, W, ZcCfg{yb, jbeg, jend, cta0});
     return cudaGetLastError();
   };
-  // 8 epilogue warps (2 column groups of 16).  16 warps (4 groups of 8) leave
-  // room for only two operand stages next to the staged Y and were slower.
-  constexpr int T8 = ZcGeo<8>::THREADS;
-  // Jobs are taken in heavy/light pairs by the small class's four-stage
-  // variant (every block and atom A of at most 16 AOs) and by both variants
-  // of the large-block class; the small class's fallbacks, for cells whose
-  // staged Y does not fit next to four stages, keep one job at a time.
-  if (P.kbmax <= 16) {
-    if (ZC_STAGE_Y && smem_of(4, 16, P.ybytes, 2) <= kMax) {
-      if (small) return launch(k_zc<KS, 16, 4, 8, true, true>, T8, 4, 16, P.ybytes, 2);
-      return launch(k_zc<KS, 16, 4, 8, true, false>, T8, 4, 16, P.ybytes, 2);
-    }
-    if (ZC_STAGE_Y && smem_of(3, 16, P.ybytes, 2) <= kMax)
-      return launch(k_zc<KS, 16, 3, 8, true, false>, T8, 3, 16, P.ybytes, 2);
-    return launch(k_zc<KS, 16, 3, 8, false, false>, T8, 3, 16, 0, 2);
-  }
-  if (ZC_STAGE_Y && smem_of(2, 32, P.ybytes, 2) <= kMax)
-    return launch(k_zc<KS, 32, 2, 8, true, true>, T8, 2, 32, P.ybytes, 2);
-  return launch(k_zc<KS, 32, 2, 8, false, true>, T8, 2, 32, 0, 2);
+  if (smem_of(4, ybytes) <= kMax) return launch(k_zc<KS, 4, 8, true, true>, 4, ybytes);
+  if (smem_of(3, ybytes) <= kMax) return launch(k_zc<KS, 3, 8, true, false>, 3, ybytes);
+  return launch(k_zc<KS, 3, 8, false, false>, 3, 0);
 }
 
-// The wave's small-class jobs [0, nsmall) with the shape of blocks of at most
-// 16 AOs, then the others with the system's shape.
+// Staged Y bytes of one block (al rows spanned by 128 (al, a) rows, all b, 2
+// pairs of padding per al) for jobs of atoms of at most 16 AOs.
+int zc_ybytes(uint64_t present) {
+  int lo = 0, hi = 0;
+  for (int n = 1; n <= 16; ++n)
+    if ((present >> n) & 1) {
+      if (!lo) lo = n;
+      hi = n;
+    }
+  return lo ? (127 / lo + 2) * (hi * 16 + ZC_YPAD) * 8 : 0;
+}
+
+// The wave's small-class jobs [0, nsmall), then the others with k_zcw.
 template <int KS>
 cudaError_t zc_run_t(const SplitShared &S, const SplitWave &W, const ZcPlanShape &P, int nsm,
                      int nsmall, cudaStream_t st) {
   const int njobs = (int)W.h_zc_jobs;
   if (nsmall > 0) {
-    const ZcPlanShape Q{16, 16, P.ybytes_small, P.ybytes_small};
-    cudaError_t e = zc_range_t<KS>(S, W, Q, nsm, 0, nsmall, 0, true, st);
+    cudaError_t e = zc_range_t<KS>(S, W, P.ybytes_small, nsm, 0, nsmall, 0, st);
     if (e != cudaSuccess) return e;
   }
   if (njobs > nsmall)
-    return zc_range_t<KS>(S, W, P, nsm, nsmall, njobs, nsm, false, st);
+    return split_zcw_run(S, W, KS, P.ybytes_wide, nsm, nsmall, njobs, nsm, st);
   return cudaSuccess;
 }
 
@@ -1364,7 +1138,9 @@ cudaError_t dz_prepare_t(const SplitShared &S, cudaStream_t st) {
 template <int KS>
 cudaError_t slice_cz_t(const SplitShared &S, cudaStream_t st) {
   if (S.h_cz_rows > 0)
-    k_slice_cz<KS><<<(unsigned)((S.h_cz_rows * 32 + 255) / 256), 256, 0, st>>>(S);
+    k_slice_cz<KS><<<(unsigned)((S.h_cz_rows * 32 + 255) / 256), 256, 0, st>>>(S, 0);
+  if (S.h_czw_rows > 0)
+    k_slice_cz<KS><<<(unsigned)((S.h_czw_rows * 32 + 255) / 256), 256, 0, st>>>(S, 1);
   return cudaGetLastError();
 }
 
@@ -1374,6 +1150,10 @@ cudaError_t split_zc_plan(const SplitShared &S, const SplitWave &W, int fill, cu
   if (W.nw <= 0) return cudaSuccess;
   split::k_zc_plan<<<(unsigned)((W.nw + 3) / 4), 128, 0, st>>>(S, W, fill);
   return cudaGetLastError();
+}
+
+ZcPlanShape split_zc_shape(uint64_t present) {
+  return ZcPlanShape{split::zc_ybytes(present), split_zcw_ybytes(present)};
 }
 
 cudaError_t split_zc_run(const SplitShared &S, const SplitWave &W, int ks, const ZcPlanShape &P,

@@ -1,0 +1,249 @@
+// Device code shared by the two kernels of the D_FG / D_FB products: k_zc for
+// blocks of at most 16 AOs (hfx_zc.cu) and k_zcw for wider ones (hfx_zcw.cu).
+#pragma once
+
+#include <cuda_bf16.h>
+
+#include <algorithm>
+
+#include "hfx_split.h"
+#include "split_common.cuh"
+
+namespace split {
+
+constexpr int ZC_COLS = 32;                      // Z columns per job
+constexpr long long ZC_WAIT = 2000000000ll;      // cycles per bounded wait
+
+// Job handed to CTA b in round r of the persistent loop: rounds alternate
+// direction (snake order), so over a longest-first list every CTA gets a
+// similar mix of long and short jobs.  The last round is partial.
+__device__ __forceinline__ int zc_job_of(int r, int b, int G) {
+  return r * G + ((r & 1) ? G - 1 - b : b);
+}
+
+// Epilogue data of one job, written to shared memory by a few lanes when its
+// pair starts and read by every epilogue thread on each of the job's tiles.
+struct ZcEpiJob {
+  int64_t y2off;     // the work item's Y pairs in the wave scratch
+  int64_t sg[2][2];  // block q: Sigma offset of its outputs, of their mirror (-1: none)
+  int pA, na, nb, mtz, nblk, R0b;
+  int nout[2], ncv[2], pc[2], gcb[2];
+  int64_t czrow0;        // first row of atom A's C exponents
+  int u, ush, slots, q;  // the A operand's rows (ZcRows, wide operand), u = 2^ush
+  int inv;          // x / na = x inv >> 16 for x < 2048
+  int ncb0;  // 16-column blocks of Y of block 0 (block 1's follow them in a staged buffer)
+};
+
+// Number of jobs CTA b receives from zc_job_of over a list of njobs.
+__device__ __forceinline__ int zc_cta_jobs(int njobs, int b, int G) {
+  const int full = njobs / G, rem = njobs - full * G;
+  return full + (((full & 1) ? G - 1 - b : b) < rem ? 1 : 0);
+}
+
+// Tile order of a CTA.  Its jobs r = 0 .. n - 1 run heaviest first (operand
+// stages x row tiles); pair p is job n - 1 - p (light) and job p (heavy), and
+// their row tiles alternate while both have some: the MMAs of a long tile then
+// run beside the epilogue of a short one, where one job after the other leaves
+// the epilogue idle through the long tiles and the tensor pipe idle through
+// the short ones.  Without PAIR, pair p is job p alone.  Every role walks the
+// same order.
+template <bool PAIR>
+struct ZcPair {
+  int r0, r1, m0, m1, t0, t1, last;
+  bool two;
+  __device__ __forceinline__ void begin(int p, int n) {
+    r0 = PAIR ? n - 1 - p : p;
+    r1 = PAIR ? p : -1;
+    two = PAIR && r1 < r0;
+    m0 = m1 = t0 = t1 = 0;
+    last = 1;
+  }
+  // next tile: job x of the pair (0: r0, 1: r1) and its row tile mt
+  __device__ __forceinline__ bool next(int &x, int &mt) {
+    const bool a = t0 < m0, b = t1 < m1;
+    if (!a && !b) return false;
+    x = (a && (!b || last == 1)) ? 0 : 1;
+    last = x;
+    mt = x ? t1++ : t0++;
+    return true;
+  }
+};
+
+template <class T>
+__device__ __forceinline__ void zc_swap(T &a, T &b) {
+  const T t = a;
+  a = b;
+  b = t;
+}
+
+__device__ __forceinline__ ZcJob zc_job(const SplitWave &W, int jbeg, int r) {
+  return W.zc_jobs[jbeg + zc_job_of(r, blockIdx.x, gridDim.x)];
+}
+
+// rows of a job's lone column block (16 or 32); two blocks have 16 each
+__device__ __forceinline__ int zc_rows(const SplitShared &S, const ZcJob &jb, const WorkItem &it) {
+  if (jb.nblk != 1) return 16;
+  const int ncb = jb.piece[0] == 1 ? S.nao[S.nbr[it.gbase + jb.g[0]].other] : S.nao[it.b];
+  return ncb <= 16 ? 16 : 32;
+}
+
+// block and first column cq of column group q of width CW: two 16-column
+// blocks take half the groups each; one block takes the groups below its R
+template <int CW>
+__device__ __forceinline__ int zc_group_block(int nblk, int R0b, int q, int &cq) {
+  const int jc = q * CW;
+  if (nblk == 2) { cq = jc & 15; return jc >> 4; }
+  cq = jc;
+  return jc < R0b ? 0 : -1;
+}
+
+// Epilogue data of job r, by one whole warp: lanes 0 .. 3 look up the Sigma
+// offsets of block lane / 2 (odd lanes: the mirror), lane 4 the scalars.  A
+// missing Sigma key fails the build, and the block is not added.
+template <bool WIDE>
+__device__ __forceinline__ void zc_epi_job(const SplitShared &S, const SplitWave &W, int jbeg,
+                                           int r, int lane, ZcEpiJob &e) {
+  const ZcJob jb = zc_job(W, jbeg, r);
+  const WorkItem it = S.items[jb.w];
+  const int q = (lane >> 1) & 1, m = lane & 1;
+  int64_t t = -1;
+  bool miss = false;
+  if (lane < 4 && q < jb.nblk) {
+    const int pcb = q ? jb.piece[1] : jb.piece[0];
+    const bool mir = S.sym && (pcb == 2 || it.role == 1);
+    if (m == 0 || mir) {
+      if (pcb == 1) {
+        t = m == 0 ? dh_find(S.shash, hk_pack(it.a, it.b, it.n[0], it.n[1], it.n[2]))
+                   : dh_find(S.shash, hk_pack(it.b, it.a, -it.n[0], -it.n[1], -it.n[2]));
+      } else {
+        const NbrEntry eg = S.nbr[it.gbase + (q ? jb.g[1] : jb.g[0])];
+        const int n0 = it.n[0] + eg.n[0], n1 = it.n[1] + eg.n[1], n2 = it.n[2] + eg.n[2];
+        t = m == 0 ? dh_find(S.shash, hk_pack(it.a, eg.other, n0, n1, n2))
+                   : dh_find(S.shash, hk_pack(eg.other, it.a, -n0, -n1, -n2));
+      }
+      miss = t < 0;
+      if (miss) atomicOr(S.err, HFX_DEV_ERR_MISSING);
+    }
+  }
+  const bool bad = __shfl_sync(0xffffffffu, (int)miss, lane & ~1) |
+                   __shfl_sync(0xffffffffu, (int)miss, lane | 1);
+  if (lane < 4) e.sg[q][m] = bad ? -1 : t;
+  if (lane == 4) {
+    const int pA = S.nabf[it.a], na = S.nao[it.a], nb = S.nao[it.b];
+    e.y2off = W.y2_off[(int)(jb.w - W.w0)];
+    e.pA = pA;
+    e.na = na;
+    e.nb = nb;
+    const ZcRows R = zc_rows_of(na);
+    e.u = R.u;
+    e.ush = __ffs(R.u) - 1;
+    e.slots = R.slots;
+    e.q = R.q;
+    e.inv = (65536 + na - 1) / na;
+    e.mtz = WIDE ? zc_tiles(pA, na) : (pA * na + 127) / 128;
+    e.czrow0 = (WIDE ? S.czw_rowpre : S.cz_rowpre)[it.a];
+    e.nblk = jb.nblk;
+    e.R0b = 16;
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      e.nout[b] = e.ncv[b] = e.pc[b] = e.gcb[b] = 0;
+      if (b < jb.nblk) {
+        const int ng = S.nao[S.nbr[it.gbase + jb.g[b]].other];
+        e.pc[b] = jb.piece[b];
+        e.gcb[b] = S.kofs[it.gbase + jb.g[b]] / 16;
+        e.ncv[b] = jb.piece[b] == 1 ? ng : nb;
+        e.nout[b] = jb.piece[b] == 1 ? nb : ng;
+      }
+    }
+    if (jb.nblk > 0) e.R0b = e.ncv[0] <= 16 ? 16 : 32;
+    e.ncb0 = jb.nblk > 0 ? (S.nao[S.nbr[it.gbase + jb.g[0]].other] + 15) / 16 : 0;
+  }
+}
+
+// Column exponents of job r's column group hf (CW columns), by lanes < CW.
+template <int CW>
+__device__ __forceinline__ void zc_epi_ecol(const SplitShared &S, const SplitWave &W, int jbeg,
+                                            int r, int hf, int lane, int *ecol) {
+  if (lane >= CW) return;
+  const ZcJob jb = zc_job(W, jbeg, r);
+  const WorkItem it = S.items[jb.w];
+  int ncv0 = 0, R0b = 16;
+  if (jb.nblk > 0) {
+    ncv0 = jb.piece[0] == 1 ? S.nao[S.nbr[it.gbase + jb.g[0]].other] : S.nao[it.b];
+    R0b = ncv0 <= 16 ? 16 : 32;
+  }
+  int c0 = 0;
+  const int hb = zc_group_block<CW>(jb.nblk, R0b, hf, c0);
+  int e = -1000;
+  if (hb >= 0) {
+    const int pc = hb ? jb.piece[1] : jb.piece[0], g = hb ? jb.g[1] : jb.g[0];
+    const int at = pc == 1 ? S.nbr[it.gbase + g].other : it.b;
+    const int ncvh = S.nao[at];  // piece 1: nao(G); piece 2: nao(B)
+    const int cc = c0 + lane;
+    if (cc < ncvh) e = row_exponent((long long)S.de[S.aoff[at] + cc]);
+  }
+  ecol[hf * CW + lane] = e;
+}
+
+// A launch's shared bytes of one staged Y buffer and its range of the job list.
+struct ZcCfg {
+  int ybytes;
+  int jbeg, jend;
+  int cta0;  // first slot of its CTAs' busy times
+};
+
+// Y rows al in [al0, al0 + nal) of the 16-column block cb: [al][b][16] pairs.
+__device__ __forceinline__ const float2 *zc_y_global(const float2 *Y2, int cb, int pA, int nb,
+                                                     int al) {
+  return Y2 + (((int64_t)cb * pA + al) * nb) * 16;
+}
+
+// One operand stage's MMAs (K = 16): for each block b, A digit i times the
+// block's B digits 0 .. KS - 1 - i stacked along N (N = R (KS - i)) into TMEM
+// columns b 16 KS + i R ..  Descriptors are the stage's two base descriptors
+// plus constant offsets (the 14-bit start field cannot carry: shared
+// addresses stay below 2^18).
+template <int KS>
+__device__ __forceinline__ void zc_stage_mmas(uint32_t a0, uint32_t b0, uint32_t dcol, int nblk,
+                                              int R, const uint32_t (&id16)[KS],
+                                              const uint32_t (&id32)[KS], bool first) {
+  const uint64_t adesc = umma::smem_desc(a0, 128, 256);
+  const uint64_t bdesc = umma::smem_desc(b0, 128, 256);
+  for (int b = 0; b < nblk; ++b) {
+    const uint64_t bd = bdesc + (uint64_t)((b * (KS * 16 * 16 * 2)) >> 4);
+#pragma unroll
+    for (int i = 0; i < KS; ++i) {
+      const uint64_t ad = adesc + (uint64_t)((i * (128 * 16 * 2)) >> 4);
+      umma::mma_bf16(dcol + (uint32_t)(b * 16 * KS + i * R), ad, bd, R == 16 ? id16[i] : id32[i],
+                     (!first || i) ? 1u : 0u);
+    }
+  }
+}
+
+// Loader-warp view of a job: operand bases, its entries (lane l holds entry
+// held + l) and the B rows per block.
+struct ZcLd {
+  const __nv_bfloat16 *A;
+  int64_t ktot, ent;
+  int nent, nblk, Rl, mtz, held;
+  ZcEnt mine;
+};
+
+template <bool WIDE>
+__device__ __forceinline__ void zc_ld_job(const SplitShared &S, const SplitWave &W, int jbeg,
+                                          int r, ZcLd &L) {
+  const ZcJob jb = zc_job(W, jbeg, r);
+  const WorkItem it = S.items[jb.w];
+  L.A = S.cz + (WIDE ? S.czw_base : S.cz_base)[it.a];
+  L.ktot = S.ktotZ[it.a];
+  L.ent = jb.ent;
+  L.nent = jb.nent;
+  L.nblk = jb.nblk;
+  L.Rl = zc_rows(S, jb, it);
+  L.mtz = WIDE ? zc_tiles(S.nabf[it.a], S.nao[it.a])
+               : (S.nabf[it.a] * S.nao[it.a] + 127) / 128;
+  L.held = -1;
+  L.mine = ZcEnt{0, {-1, -1}};
+}
+
+}  // namespace split
