@@ -392,7 +392,7 @@ hfx_status pack_kind(hfx_ctx *ctx, int k) {
   CK(K.d_offs.reserve(nblk + 1));
   CK(cudaMemcpyAsync(K.d_offs.p, K.offs.data(), sizeof(int64_t) * (nblk + 1),
                      cudaMemcpyHostToDevice, st));
-  CK(K.maxabs.reserve(nblk));
+  CK(K.maxabs.reserve(nblk + 1));
   CK(launch_maxabs(K.data.p, K.d_offs.p, nblk, K.maxabs.p, ctx->d_err.p, st));
   ctx->launches += nblk > 0;
   K.dirty = false;
@@ -1130,6 +1130,7 @@ hfx_status hfx_build(hfx_ctx *ctx, double theta, hfx_prec prec, int32_t nslices,
     a.C = DevBlocks{ctx->K[0].data.p, ctx->K[0].d_offs.p, ctx->K[0].maxabs.p};
     a.V = DevBlocks{ctx->K[1].data.p, ctx->K[1].d_offs.p, ctx->K[1].maxabs.p};
     a.D = DevBlocks{ctx->K[2].data.p, ctx->K[2].d_offs.p, ctx->K[2].maxabs.p};
+    a.nD = (int64_t)ctx->K[2].keys.size();
     a.dhash = DevHash{ctx->d_dhkeys.p, ctx->d_dhvals.p, ctx->dmask};
     a.theta = theta;
     a.masks = ctx->d_masks.p;

@@ -129,6 +129,7 @@ struct ScreenArgs {
   const NbrEntry *nbr;
   const int32_t *nao, *nabf;
   DevBlocks C, V, D;
+  int64_t nD;              // D blocks; D.maxabs[nD] is the largest of all
   DevHash dhash;
   double theta;
   uint32_t *masks;
@@ -176,6 +177,7 @@ struct ContractArgs {
   double *dv;                // adjoint: dE/dV in the V block layout
 };
 
+// out[e] = max|x| of block e, out[nblk] that of all of them (zeroed here first).
 cudaError_t launch_maxabs(const double *data, const int64_t *offs, int64_t nblk, double *out,
                           unsigned *err, cudaStream_t st);
 cudaError_t launch_screen(const ScreenArgs &a, cudaStream_t st);

@@ -1,7 +1,7 @@
 // Block upper limits and the per-term screen (Sec. III.B-C of the paper).
 //
 //  * k_maxabs: max|x| of every block (the upper limit of Sec. III.B), one warp
-//    per block; flags NaN/Inf.
+//    per block, and of all blocks together; flags NaN/Inf.
 //  * k_screen: one warp per (work item <A,B>, G in N[B]).  For every F in N[A]
 //    and each of the four placements of the ABF centres (Algorithm 2/3:
 //    D_FG -> Sigma_AB, D_FB -> Sigma_AG, D_AG -> Sigma_FB, D_AB -> Sigma_FG)
@@ -10,6 +10,10 @@
 //    S > theta (strict, as Algorithm 4).  With the Cauchy-Schwarz ERI screen
 //    on (Sec. III.C, Eq. CS-ERI) a quadruple (A,B,F,G) also needs
 //    sqrt(Q_AF) sqrt(Q_BG) > eps_eri, else all four of its terms go.
+//    Most F fall to the largest D block of all: if S with it fails, S with any
+//    D does (rounded products keep the order), so no D block is looked up.  The
+//    lookups were most of the kernel; as N[A] runs by descending max|C|, the
+//    first 32 F that all fall end the row.
 //    Survivors become bits of four F-bitmasks per (A,B,G); their Sigma keys go
 //    into a hash set.
 //  * k_diag_eri: one block per C block, the largest diagonal ERI Q of its AO
@@ -32,7 +36,11 @@ __global__ void k_maxabs(const double *__restrict__ data, const int64_t *__restr
   }
   for (int o = 16; o; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
   if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(err, HFX_DEV_ERR_NONFINITE);
-  if (lane == 0) out[warp] = m;
+  if (lane == 0) {
+    out[warp] = m;
+    // nonnegative doubles order as their bit patterns
+    atomicMax((unsigned long long *)(out + nblk), (unsigned long long)__double_as_longlong(m));
+  }
 }
 
 // u^T V w over one V block ([nu][nw] row-major, nullptr = absent), with u and
@@ -151,12 +159,25 @@ __global__ void __launch_bounds__(256, 3) k_screen(ScreenArgs A) {
   const double sqBG = A.eri_sq ? A.eri_sq[eg.cblk] : 0.0;
   unsigned any = 0;
   uint32_t *mrow = A.masks + it.mask_off + (int64_t)g * 4 * it.nFw;
+  const double mvD = __dmul_rn(mv, A.D.maxabs[A.nD]);  // with the largest D block
+  bool done = false;
   for (int f0 = 0; f0 < it.nF; f0 += 32) {
     const int f = f0 + lane;
-    bool b1 = false, b2 = false, b3 = false, b4 = false;
+    bool b1 = false, b2 = false, b3 = false, b4 = false, low = true;
     int ft = 0, mF0 = 0, mF1 = 0, mF2 = 0, nf = 0;
+    NbrEntry ef;
+    if (f < it.nF && !done) {
+      ef = A.nbr[it.fbase + f];
+      low = !(__dmul_rn(__dmul_rn(A.C.maxabs[ef.cblk], mcBG), mvD) > theta);
+    }
+    // every F of the word falls, and so do the smaller ones after it; the ERI
+    // screen still counts them
+    if (!A.eri_sq && (done || __all_sync(0xffffffffu, low))) {
+      done = true;
+      if (lane < 4) mrow[lane * it.nFw + (f0 >> 5)] = 0;
+      continue;
+    }
     if (f < it.nF) {
-      const NbrEntry ef = A.nbr[it.fbase + f];
       ft = ef.other; mF0 = ef.n[0]; mF1 = ef.n[1]; mF2 = ef.n[2];
       nf = A.nao[ft];
       const bool f_is_a = (ft == it.a) && mF0 == 0 && mF1 == 0 && mF2 == 0;
@@ -164,7 +185,7 @@ __global__ void __launch_bounds__(256, 3) k_screen(ScreenArgs A) {
       // the Cauchy-Schwarz ERI screen removes the whole quadruple
       const bool eri_ok = !A.eri_sq || __dmul_rn(A.eri_sq[ef.cblk], sqBG) > A.eps_eri;
       eri_cut += eri_ok ? 0 : 1;
-      if (eri_ok) {
+      if (eri_ok && !low) {
         // variant 1: D_FG -> Sigma_AB
         const int64_t dFG = dfind(A.dhash, ft, gt, nG0 - mF0, nG1 - mF1, nG2 - mF2);
         if (dFG >= 0) b1 = __dmul_rn(cc, __dmul_rn(mv, A.D.maxabs[dFG])) > theta;
@@ -250,6 +271,8 @@ __global__ void k_collect_keys(const unsigned long long *keys, uint64_t cap,
 cudaError_t launch_maxabs(const double *data, const int64_t *offs, int64_t nblk, double *out,
                           unsigned *err, cudaStream_t st) {
   if (nblk <= 0) return cudaSuccess;
+  cudaError_t e = cudaMemsetAsync(out + nblk, 0, sizeof(double), st);
+  if (e != cudaSuccess) return e;
   const int64_t threads = nblk * 32;
   k_maxabs<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(data, offs, nblk, out, err);
   return cudaGetLastError();
