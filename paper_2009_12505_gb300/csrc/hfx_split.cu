@@ -265,26 +265,35 @@ __global__ void __launch_bounds__(PD_THREADS, 3) k_pdig(SplitShared S, SplitWave
     for (int idx = threadIdx.x; idx < gn * KT8; idx += PD_THREADS) {
       const int gi = idx / KT8, c8 = (idx - gi * KT8) * 8;
       const int e = es[gi];
-      // scale by 2^(7 KS - e) (|value| < 2^(e - 1)) in two exact steps
-      const int sft = 7 * KS - e, s1 = sft / 2, s2 = sft - s1;
-      const float f1 = __int_as_float((s1 + 127) << 23), f2 = __int_as_float((s2 + 127) << 23);
+      // scaled by 2^(6 - e) in two exact steps (|value| < 2^(e - 1)), digit s is a
+      // multiple of 2^(-7 s): adding and taking away 1.5 2^(23 - 7 s) rounds to
+      // it and leaves the exact rest (f32 only: the 64-bit conversions ran on the
+      // FP64 pipe).  Below 2^-200 the row is dropped.
+      const int sft = e > -200 ? 7 - e : 0, s1 = sft / 2, s2 = sft - s1;
+      const float q1 = e > -200 ? __int_as_float((s1 + 127) << 23) : 0.f;
+      const float q2 = __int_as_float((s2 + 127) << 23);
+      const uint64_t f1 = f2_pk(q1, q1), f2 = f2_pk(q2, q2);
       uint32_t pk[KS][4];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const int c = c8 + k;
-        long long X = 0;
-        if (c < K && e > -200) {  // below 2^-200 the row is dropped
-          const float2 v = Ps[gi * K + c];
-          X = __float2ll_rn(__fmul_rn(__fmul_rn(v.x, f1), f2)) +
-              __float2ll_rn(__fmul_rn(__fmul_rn(v.y, f1), f2));
-        }
-        int d[KS];
-        to_digits_i64<KS>(X, d);
+      for (int k = 0; k < 4; ++k) {
+        const int c = c8 + 2 * k;
+        const float2 z = make_float2(0.f, 0.f);
+        const float2 u = c < K ? Ps[gi * K + c] : z, v = c + 1 < K ? Ps[gi * K + c + 1] : z;
+        // renormalised, so the low words are below the third digit
+        uint64_t h = 0, l = 0;
+        df_acc2(h, l, f2_mul(f2_mul(f2_pk(u.x, v.x), f1), f2));
+        df_acc2(h, l, f2_mul(f2_mul(f2_pk(u.y, v.y), f1), f2));
 #pragma unroll
         for (int sd = 0; sd < KS; ++sd) {
-          const uint32_t b = __bfloat16_as_ushort(__int2bfloat16_rn(d[sd]));
-          if (k & 1) pk[sd][k >> 1] |= b << 16;
-          else pk[sd][k >> 1] = b;
+          // digit as a whole number: 2^(7 sd) times the multiple
+          const float m = __int_as_float((23 - 7 * sd + 127) << 23 | 0x400000);
+          const float w = __int_as_float((7 * sd + 127) << 23);
+          const uint64_t M = f2_pk(m, m);
+          const uint64_t t = f2_sub(f2_add(h, M), M);
+          h = f2_sub(h, t);
+          if (sd == 2) h = f2_add(h, l);
+          const float2 d = f2_un(f2_mul(t, f2_pk(w, w)));
+          asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(pk[sd][k]) : "f"(d.y), "f"(d.x));
         }
       }
       const int r = eg.aopre + g0 + gi;
