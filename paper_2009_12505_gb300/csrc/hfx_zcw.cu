@@ -241,10 +241,12 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
   if (warp == ZC_EPI) {
     // ------------------------------------------------------------ A / B loader
     // the whole warp walks the steps.  Lane l holds entry q0 + l of the job
-    // (fetched 32 at a time, off the per-stage path); lane 0 waits and arms
-    // the stage, then lane 0 copies the A tile and lanes 1 .. nblk one whole
-    // B block each
-    long long step = 0;
+    // (fetched 32 at a time, off the per-stage path) and waits for its stage,
+    // arms it and issues its copies itself, so a stage costs no shuffles; the
+    // lanes take turns, as the ring's parities need the stages in order
+    int s = 0;           // the ring's slot and the parity of its last release
+    uint32_t ph = 1;     // (the first round waits for none)
+    int step = 0, last = -1;  // stages passed, the last one this lane armed
     bool ok = true;
     for (int p = 0; p < npair && ok; ++p) {
       // one decision for the whole warp
@@ -264,56 +266,50 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
           zc_swap(L, Lo);
           cur = x;
         }
-        const int cb = lane - 1;
-        const bool has_b = lane >= 1 && lane <= L.nblk;
+        const uint32_t bb = (uint32_t)(KS * 16 * 2) * (uint32_t)L.Rl;  // bytes of a B block
         for (int q0 = 0; q0 < L.nent && ok; q0 += 32) {
           if (L.held != q0) {
             if (q0 + lane < L.nent) L.mine = W.zc_ents[L.ent + q0 + lane];
             L.held = q0;
           }
           const int nq = min(32, L.nent - q0);
-          for (int qq = 0; qq < nq; ++qq, ++step) {
-            const int kofs = __shfl_sync(0xffffffffu, L.mine.kofs, qq);
-            const long long d0 = __shfl_sync(0xffffffffu, (long long)L.mine.dz[0], qq);
-            const long long d1 = __shfl_sync(0xffffffffu, (long long)L.mine.dz[1], qq);
-            const int s = (int)(step % NST);
-            bool w = true;
-            if (lane == 0) {
-              if (step >= NST)
-                w = umma::mbar_wait(&ctl->empty[s], (uint32_t)((step / NST - 1) & 1), S.err,
-                                    ZC_WAIT);
-              w = w && !*abort_f;
+          const __nv_bfloat16 *a = L.A + ((int64_t)mt * L.ktot + L.mine.kofs) * KS * 128;
+          const __nv_bfloat16 *b0 = L.mine.dz[0] >= 0 ? S.dz + L.mine.dz[0] : S.dzero;
+          const __nv_bfloat16 *b1 = L.mine.dz[1] >= 0 ? S.dz + L.mine.dz[1] : S.dzero;
+          for (int qq = 0; qq < nq; ++qq) {
+            if (lane == qq) {
+              // once the build is given up, a stage that is not free stays so
+              ok = step < NST || umma::mbar_try_wait(&ctl->empty[s], ph) ||
+                   (!*abort_f && umma::mbar_wait(&ctl->empty[s], ph, S.err, ZC_WAIT));
+              if (!ok) {
+                *abort_f = 1;
+              } else {
+                last = step;
+                uint8_t *st = smem + s * STG;
+                umma::mbar_arrive_expect_tx(&ctl->full[s], A_BYTES + bb * (uint32_t)L.nblk);
+                umma::bulk_g2s(st, a, A_BYTES, &ctl->full[s]);
+                // B stage block-major: block b's KS digits of Rl rows x 16 K at b KS 16 16
+                umma::bulk_g2s(st + A_BYTES, b0, bb, &ctl->full[s]);
+                if (L.nblk > 1)
+                  umma::bulk_g2s(st + A_BYTES + KS * 16 * 16 * 2, b1, bb, &ctl->full[s]);
+              }
             }
-            w = __shfl_sync(0xffffffffu, (int)w, 0) != 0;
-            if (!w) {
-              if (lane == 0) *abort_f = 1;
-              ok = false;
-              break;
-            }
-            uint8_t *st = smem + s * STG;
-            const uint32_t bbytes = (uint32_t)(KS * 16 * 2) * (uint32_t)(L.nblk * L.Rl);
-            if (lane == 0) umma::mbar_arrive_expect_tx(&ctl->full[s], A_BYTES + bbytes);
             __syncwarp();
-            if (lane == 0) {
-              umma::bulk_g2s(st, L.A + ((int64_t)mt * L.ktot + kofs) * KS * 128, A_BYTES,
-                             &ctl->full[s]);
-            } else if (has_b) {
-              // B stage block-major: block b's KS digits of Rl rows x 16 K at b KS 16 16
-              const int64_t dz = cb == 0 ? d0 : d1;
-              const __nv_bfloat16 *src = dz >= 0 ? S.dz + dz : S.dzero;
-              umma::bulk_g2s(st + A_BYTES + cb * (KS * 16 * 16 * 2), src,
-                             (uint32_t)(KS * L.Rl * 16 * 2), &ctl->full[s]);
+            ++step;
+            if (++s == NST) {
+              s = 0;
+              ph ^= 1;
             }
           }
+          ok = __all_sync(0xffffffffu, ok);
         }
       }
     }
     // drain: the last stages issued must have landed before the CTA exits
-    if (lane == 0) {
-      const long long first = step > NST ? step - NST : 0;
-      for (long long t = first; t < step; ++t)
+    last = __reduce_max_sync(0xffffffffu, last);
+    if (lane == 0)
+      for (int t = max(0, last + 1 - NST); t <= last; ++t)
         umma::mbar_wait(&ctl->full[t % NST], (uint32_t)((t / NST) & 1), S.err, ZC_WAIT);
-    }
   } else if (warp >= ZC_EPI + 2) {
     // ------------------------------------------------------------ Y warps
     // the first copies each tile's Y rows (and its row exponents) into a shared
@@ -404,7 +400,9 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
   } else if (warp == ZC_EPI + 1) {
     // ------------------------------------------------------------ MMA issuer
     if (lane == 0) {
-      long long step = 0, hand = 0;
+      long long hand = 0;
+      int s = 0;  // operand slot and its parity
+      uint32_t ph = 0;
       // N = R (KS - i) for a block of R rows (16 or 32), 16 KS at most 192
       uint32_t idesc16[KS], idesc32[KS];
 #pragma unroll
@@ -447,9 +445,8 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
           }
           umma::fence_after_sync();
           const uint32_t dcol = tbase + (uint32_t)(tb * 256);
-          for (int q = 0; q < nent; ++q, ++step) {
-            const int s = (int)(step % NST);
-            if (!umma::mbar_wait(&ctl->full[s], (uint32_t)((step / NST) & 1), S.err, ZC_WAIT)) {
+          for (int q = 0; q < nent; ++q) {
+            if (!umma::mbar_wait(&ctl->full[s], ph, S.err, ZC_WAIT)) {
               ok = false;
               break;
             }
@@ -457,6 +454,10 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
             const uint32_t a0 = sbase + (uint32_t)(s * STG);
             zc_stage_mmas<KS>(a0, a0 + A_BYTES, dcol, nblk, R, idesc16, idesc32, q == 0);
             umma::mma_commit(&ctl->empty[s]);
+            if (++s == NST) {
+              s = 0;
+              ph ^= 1;
+            }
           }
           if (!ok) break;
           umma::mma_commit(&ctl->tfull[tb]);
