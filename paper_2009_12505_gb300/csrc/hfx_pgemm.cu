@@ -7,7 +7,7 @@
 // every digit-order group sum stays an exact f32 integer), and the epilogue
 // adds up the chunks before it writes the tile once: in int64 for D_AB, in
 // packed double-float for Y (whose result is an f32 pair anyway):
-//   Y job:    rows (b, G, g) of C_B transposed, columns al of V_AB, K = beta;
+//   Y job:    rows (G, b, g) of C_B transposed, columns al of V_AB, K = beta;
 //   D_AB job: rows (F, f) of C_A, columns (G, g) of P, K = (al, a).
 // Both operands are stored as KS balanced base-128 bf16 digits, one exponent
 // per row; the B digits of a K tile are contiguous, so one MMA with A digit i
@@ -66,6 +66,7 @@ struct PgMetaY {
   int64_t y2base;     // scratch offset (doubles) of the pair's Y2 region
   int64_t y64base;    // scratch offset of the pair's FP64 Y region
   int32_t pA, nbY, nrowY, pad;
+  int32_t y64row[TM];  // row in the FP64 Y, [b][(G, g)]
   int32_t y2row[TM];  // Y2 offset (pairs) of each row, -1: the row is not stored;
                       // below 2^31: at most 512 blocks of 16 x 256 x 32 x 16 pairs
   int16_t ea[TM];     // row exponents
@@ -203,7 +204,7 @@ __device__ __noinline__ void dab_lookup(const SplitShared &S, const Job &jb, int
 
 // Fill m for Y job jb (the whole job-data warp; lane l takes rows l, l + 32,
 // l + 64, l + 96).  The loads are issued level by level for the four rows at
-// once, so the dependent chain is three loads deep, not twelve.
+// once, so the dependent chain is four loads deep, not twelve.
 __device__ __forceinline__ void y_meta_fill(const SplitShared &S, const SplitWave &W,
                                             const Job &jb, const WorkItem &it, PgMetaY &m,
                                             int lane) {
@@ -221,37 +222,39 @@ __device__ __forceinline__ void y_meta_fill(const SplitShared &S, const SplitWav
     m.nbY = nbY;
     m.nrowY = nrowY;
   }
-  int b[RPL], col[RPL], G[RPL];
+  int G[RPL];
   bool live[RPL];
   int16_t ea[RPL];
 #pragma unroll
   for (int u = 0; u < RPL; ++u) {
     const int rowY = jb.mt * TM + lane + 32 * u;
     live[u] = rowY < nrowY && W.y2_on;
-    b[u] = live[u] ? rowY / ncol : 0;
-    col[u] = live[u] ? rowY - b[u] * ncol : 0;
+    // row (G, b, g): rows aopre(G) nb .. hold G, so row / nb is one of G's columns
+    G[u] = live[u] ? S.colG[coloff + rowY / nbY] : 0;
     ea[u] = ea_p[lane + 32 * u];  // padded rows hold the slicing's exponent too
   }
-#pragma unroll
-  for (int u = 0; u < RPL; ++u) G[u] = live[u] ? S.colG[coloff + col[u]] : 0;
-  int aopre[RPL], kofs[RPL];
+  int aopre[RPL], kofs[RPL], other[RPL], ng[RPL];
   unsigned bits[RPL];
 #pragma unroll
   for (int u = 0; u < RPL; ++u) {
     aopre[u] = live[u] ? S.nbr[it.gbase + G[u]].aopre : 0;
+    other[u] = live[u] ? S.nbr[it.gbase + G[u]].other : 0;
     kofs[u] = live[u] ? S.kofs[it.gbase + G[u]] : 0;
     bits[u] = live[u] ? S.wg[it.wg_off + G[u]] : 0u;
   }
 #pragma unroll
+  for (int u = 0; u < RPL; ++u) ng[u] = S.nao[other[u]];
+  // only rows that the f32 pairs' readers need: the D_FG / D_FB products and P
+  // of the D_AB piece
+  const unsigned need = y_need(S, it) & 11u;
+#pragma unroll
   for (int u = 0; u < RPL; ++u) {
-    // only rows of G with survivors are read: the f32 pairs by the D_FG /
-    // D_FB products and by P of the D_AB piece
-    int32_t y2 = -1;
-    if (live[u] && (bits[u] & 11u)) {
-      const int g = col[u] - aopre[u];
-      y2 = (((kofs[u] / 16 + g / 16) * pA) * nbY + b[u]) * 16 + (g & 15);
-    }
-    m.y2row[lane + 32 * u] = y2;
+    const int rem = jb.mt * TM + lane + 32 * u - aopre[u] * nbY;
+    const int b = rem / ng[u], g = rem - b * ng[u];
+    m.y64row[lane + 32 * u] = b * ncol + aopre[u] + g;
+    m.y2row[lane + 32 * u] =
+        live[u] && (bits[u] & need) ? (((kofs[u] / 16 + g / 16) * pA) * nbY + b) * 16 + (g & 15)
+                                    : -1;
     m.ea[lane + 32 * u] = ea[u];
   }
   const int ncl = pA - jb.nt * NT;
@@ -480,7 +483,7 @@ __global__ void __launch_bounds__(PgGeo<JOB>::THREADS, 1) k_pgemm(SplitShared S,
       // Y: the column exponents (pairs of int16)
       uint32_t ebp[JOB == 0 ? PG_CW / 2 : 1];
       bool valid;
-      // Y job: row (b, G, g) of Y, Y2 row, FP64 need, Y regions
+      // Y job: row of the FP64 Y, Y2 row, FP64 need, Y regions
       int64_t yrow = 0, y2row = -1, nrowY = 0, y2base = 0, y64base = 0;
       bool need64 = false;
       int pA = 0, nbY = 0;
@@ -507,9 +510,8 @@ __global__ void __launch_bounds__(PgGeo<JOB>::THREADS, 1) k_pgemm(SplitShared S,
         nrowY = m.nrowY;
         y2base = m.y2base;
         y64base = m.y64base;
-        const int rowY = jb.mt * TM + row;
-        valid = rowY < nrowY;
-        yrow = rowY;
+        valid = jb.mt * TM + row < nrowY;
+        yrow = m.y64row[row];
         need64 = W.y64_mode == 1;
         y2row = m.y2row[row];
         // the slot is free for the loader once every warp has read it

@@ -2,10 +2,13 @@
 // D_AB piece of Algorithm 3, which run as exact split-precision tcgen05
 // products in hfx_pgemm.cu (hfx_ozaki.cu documents the digit scheme).
 //
-//   Y job  (one per 128 rows (b,G,g) of a work item <A,B>):
-//       Y^T[(b,G,g)][al] = sum_be C_BG[be][b][g] V_AB[al][be]
-//     A operand: C of atom B transposed (rows (b,G,g), K = be), sliced once
+//   Y job  (one per 128 rows (G,b,g) of a work item <A,B>):
+//       Y^T[(G,b,g)][al] = sum_be C_BG[be][b][g] V_AB[al][be]
+//     A operand: C of atom B transposed (rows (G,b,g), K = be), sliced once
 //     per build; B operand: V_AB (rows al, K = be), sliced once per build.
+//     G is the slowest row index: N[B] runs by descending max|C|, so the G with
+//     survivors lead and fill whole tiles (with b slowest they began again in
+//     every b: 65 tiles of a pair where 54 do, 8-atom cell).
 //   D_AB job (128 rows (F,f) x 64 columns (G,g) of a pair, K chunk <= 640):
 //       Sigma_FG[f][g] -= sum_{al,a} C_AF[al][a][f] P_G[al][a][g]
 //     A operand: C of atom A as rows (F,f), K = (al,a), sliced once per
@@ -54,20 +57,19 @@ __device__ __forceinline__ void slice_row(const Src &src, int64_t row_global, in
   }
 }
 
-// C of atom x transposed for the Y product: row (b, G, g) = b * ncol + col(G,g), K = beta.
+// C of atom x transposed for the Y product: row (G, b, g) = aopre(G) nb + b ng + g,
+// K = beta.
 struct SrcCY {
   const double *Cd;
   const int64_t *Co;
   const NbrEntry *nbr;
   const int32_t *nao;
   int64_t base;
-  int n, nb, ncol;
+  int n, nb;
   __device__ bool row_live(int) const { return true; }
   __device__ double get(int r, int beta) const {
-    const int b = r / ncol, c = r - b * ncol;
-    const NbrEntry &e = nbr[base + entry_of(nbr, base, n, c)];
-    const int ng = nao[e.other], g = c - e.aopre;
-    return Cd[Co[e.cblk] + ((int64_t)beta * nb + b) * ng + g];
+    const NbrEntry &e = nbr[base + entry_of(nbr, base, n, r / nb)];
+    return Cd[Co[e.cblk] + (int64_t)beta * nb * nao[e.other] + r - e.aopre * nb];
   }
 };
 
@@ -111,7 +113,7 @@ __global__ void k_slice_atoms(SplitShared S, int which /*0: CY, 1: C4*/) {
   const int64_t base = S.nc_start[x];
   const int n = (int)(S.nc_start[x + 1] - base);
   if (which == 0) {
-    SrcCY src{S.Cd, S.Co, S.nbr, S.nao, base, n, nx, ncol};
+    SrcCY src{S.Cd, S.Co, S.nbr, S.nao, base, n, nx};
     slice_row<KS>(src, grow, r, TM, nx * ncol, px, S.ktY[x], S.cy + S.cy_base[x], S.cy_e);
   } else {
     SrcC4 src{S.Cd, S.Co, S.nbr, S.nao, base, n};
@@ -327,23 +329,14 @@ __global__ void k_jobs_y(SplitShared S, SplitWave W) {
   const int local = (int)(t - W.y_candpre[lo]);
   const int ntv = (S.nabf[it.a] + NT - 1) / NT;
   const int mt = local / ntv, nt = local - mt * ntv;
-  // skip tiles whose rows (b, G, g) belong only to G without a surviving term
-  const int ncol = S.ncol[it.b], nrow = S.nao[it.b] * ncol;
+  // skip tiles whose rows (G, b, g) belong only to G whose Y nothing reads
+  const int nb = S.nao[it.b], nrow = nb * S.ncol[it.b];
   const int r0 = mt * TM, r1 = min(nrow, r0 + TM) - 1;
-  const int b0 = r0 / ncol, b1 = r1 / ncol;
-  const int c0 = r0 - b0 * ncol, c1 = r1 - b1 * ncol;
-  int G0 = entry_of(S.nbr, it.gbase, it.nG, c0), G1 = entry_of(S.nbr, it.gbase, it.nG, c1);
+  const int G0 = entry_of(S.nbr, it.gbase, it.nG, r0 / nb);
+  const int G1 = entry_of(S.nbr, it.gbase, it.nG, r1 / nb);
+  const unsigned need = y_need(S, it);
   bool any = false;
-  if (b1 > b0 + 1 || (b1 == b0 + 1 && G1 >= G0)) {
-    G0 = 0;
-    G1 = it.nG - 1;
-  }
-  if (b1 == b0 || G0 == 0) {
-    for (int g = G0; g <= G1 && !any; ++g) any = S.wg[it.wg_off + g] != 0;
-  } else {  // wraps: [G0, nG) then [0, G1]
-    for (int g = G0; g < it.nG && !any; ++g) any = S.wg[it.wg_off + g] != 0;
-    for (int g = 0; g <= G1 && !any; ++g) any = S.wg[it.wg_off + g] != 0;
-  }
+  for (int g = G0; g <= G1 && !any; ++g) any = (S.wg[it.wg_off + g] & need) != 0;
   W.jobs[t] = Job{W.w0 + wl, mt, nt, 0, any ? S.ktY[it.b] : 0};
   if (any) atomicAdd(W.tmacs, (unsigned long long)TM * NT * TK * S.ktY[it.b]);
 }

@@ -73,7 +73,7 @@ struct SplitShared {
   unsigned *err;
   int32_t sym;
   int32_t ks;                      // digits per operand (D tile strides)
-  // C of each atom transposed for Y: rows (b, G, g), K = beta
+  // C of each atom transposed for Y: rows (G, b, g), K = beta
   __nv_bfloat16 *cy;
   const int64_t *cy_base, *cy_rowpre;
   int16_t *cy_e;

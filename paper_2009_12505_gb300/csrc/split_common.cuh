@@ -5,6 +5,7 @@
 
 #include <cuda_bf16.h>
 
+#include "hfx_split.h"
 #include "umma.cuh"
 
 namespace split {
@@ -73,6 +74,12 @@ __device__ __forceinline__ void fx_add_scaled(unsigned long long *hi_lo, long lo
   const long long lo = (long long)(V & (__int128)0xFFFFFFFFll);
   if (hi) atomicAdd(hi_lo, (unsigned long long)hi);
   if (lo) atomicAdd(hi_lo + 1, (unsigned long long)lo);
+}
+
+// The pieces (bits of wg) that read Y of work item it: with mirror pieces no
+// D_AG piece, and on the mirror of a canonical pair the D_FB piece only.
+__device__ __forceinline__ unsigned y_need(const SplitShared &S, const WorkItem &it) {
+  return !S.sym ? 0xFu : it.role == 2 ? 2u : 11u;
 }
 
 // Index of the neighbour entry of [base, base + n) whose column range holds col.
