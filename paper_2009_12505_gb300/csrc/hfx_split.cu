@@ -154,7 +154,7 @@ constexpr int PD_THREADS = 256;
 template <int KS>
 __global__ void __launch_bounds__(PD_THREADS, 3) k_pdig(SplitShared S, SplitWave W) {
   extern __shared__ __align__(16) float2 Ps[];  // [gc][K], then the staged Y
-  __shared__ int es[32];
+  __shared__ unsigned pmax[4];    // largest |P| of each g column (bit pattern)
   __shared__ float2 Dp[32 * 32];  // D_AB as f32 pairs
   const int64_t t = blockIdx.x;
   int lo = 0, hi = W.nw - 1;
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(PD_THREADS, 3) k_pdig(SplitShared S, SplitWave
   int16_t *eout = W.ps_e + W.p_rowpre[wl];
   const float2 *Y2 = reinterpret_cast<const float2 *>(W.scratch + W.y2_off[wl]);
   const double *Dab = S.Dd + S.Do[it.dab];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31;
   for (int i = threadIdx.x; i < na * nb; i += PD_THREADS) {
     const double d = Dab[i];
     const float h = __double2float_rn(d);
@@ -187,29 +187,32 @@ __global__ void __launch_bounds__(PD_THREADS, 3) k_pdig(SplitShared S, SplitWave
   const int cap = S.pd_pairs;  // >= K + nrow for every pair (sized on the host)
   const int gc = 4 * (K + nrow) <= cap ? 4 : 2 * (K + nrow) <= cap ? 2 : 1;
   float2 *Ys = Ps + gc * K;
-  for (int g0 = 0; g0 < ng; g0 += gc) {
-    const int gn = min(gc, ng - g0);
-    // stage Y[al][b][g0 .. g0 + gc) (Y2 layout [cb][al][b][16]; g0 is a multiple
-    // of gc, so the gc pairs stay inside one 16-column block and one sector)
-    // staged as [al][b] rows of gc high words, then gc low words (gc > 1), so
-    // two columns' high (low) words are one register pair
+  // stage Y[al][b][g0 .. g0 + gc) as [al][b] rows of gc pairs (Y2 layout
+  // [cb][al][b][16]; g0 is a multiple of gc, so the gc pairs stay inside one
+  // 16-column block and one sector).  The next pass's rows are copied while
+  // this pass's digits are written: Ys is free by then.
+  auto stage = [&](int g0) {
     const float2 *yb = Y2 + ((int64_t)(cbG + (g0 >> 4)) * pA * nb) * 16 + (g0 & 15);
-    float *Yf = reinterpret_cast<float *>(Ys);
     for (int r = threadIdx.x; r < nrow; r += PD_THREADS) {
       const float2 *src = yb + (int64_t)r * 16;
-      if (gc == 4) {
-        const float4 u0 = reinterpret_cast<const float4 *>(src)[0];
-        const float4 u1 = reinterpret_cast<const float4 *>(src)[1];
-        reinterpret_cast<float4 *>(Yf + r * 8)[0] = make_float4(u0.x, u0.z, u1.x, u1.z);
-        reinterpret_cast<float4 *>(Yf + r * 8)[1] = make_float4(u0.y, u0.w, u1.y, u1.w);
-      } else if (gc == 2) {
-        const float4 u0 = reinterpret_cast<const float4 *>(src)[0];
-        reinterpret_cast<float4 *>(Yf + r * 4)[0] = make_float4(u0.x, u0.z, u0.y, u0.w);
+      const uint32_t dst = umma::smem_u32(Ys + r * gc);
+      if (gc == 1) {
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
       } else {
-        Ys[r] = src[0];
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+        if (gc == 4)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16), "l"(src + 2)
+                       : "memory");
       }
     }
+  };
+  stage(0);
+  for (int g0 = 0; g0 < ng; g0 += gc) {
+    const int gn = min(gc, ng - g0);
+    if (threadIdx.x < 4) pmax[threadIdx.x] = 0;
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
+    unsigned mx[4] = {0, 0, 0, 0};
     if (gc == 1) {
       for (int kap = threadIdx.x; kap < K; kap += PD_THREADS) {
         const int al = kap / na, a = kap - al * na;
@@ -218,13 +221,14 @@ __global__ void __launch_bounds__(PD_THREADS, 3) k_pdig(SplitShared S, SplitWave
         float sh = 0.f, sl = 0.f;
         for (int b = 0; b < nb; ++b) df_mac(sh, sl, d[b], y[b]);
         Ps[kap] = make_float2(sh, sl);
+        mx[0] = max(mx[0], __float_as_uint(fabsf(sh)));
       }
     } else {
       // all gn columns of one (al, a) per thread, two per packed (f32x2)
       // operation; each lane takes exactly the scalar df_mac's operations
       for (int kap = threadIdx.x; kap < K; kap += PD_THREADS) {
         const int al = kap / na, a = kap - al * na;
-        const float *yr = Yf + (int64_t)al * nb * 2 * gc;
+        const float4 *yr = reinterpret_cast<const float4 *>(Ys + al * nb * gc);
         const float2 *d = Dp + a * nb;
         uint64_t s0 = 0, r0 = 0, s1 = 0, r1 = 0;
         for (int b = 0; b < nb; ++b) {
@@ -232,13 +236,12 @@ __global__ void __launch_bounds__(PD_THREADS, 3) k_pdig(SplitShared S, SplitWave
           const uint64_t ah = f2_pk(dv.x, dv.x), nah = f2_pk(-dv.x, -dv.x),
                          nal = f2_pk(-dv.y, -dv.y);
           if (gc == 4) {
-            const float4 H = reinterpret_cast<const float4 *>(yr + b * 8)[0];
-            const float4 L = reinterpret_cast<const float4 *>(yr + b * 8)[1];
-            df_mac2(s0, r0, ah, nah, nal, f2_pk(H.x, H.y), f2_pk(L.x, L.y));
-            df_mac2(s1, r1, ah, nah, nal, f2_pk(H.z, H.w), f2_pk(L.z, L.w));
+            const float4 u = yr[2 * b], v = yr[2 * b + 1];  // (h, l) of two columns each
+            df_mac2(s0, r0, ah, nah, nal, f2_pk(u.x, u.z), f2_pk(u.y, u.w));
+            df_mac2(s1, r1, ah, nah, nal, f2_pk(v.x, v.z), f2_pk(v.y, v.w));
           } else {
-            const float4 V = reinterpret_cast<const float4 *>(yr + b * 4)[0];
-            df_mac2(s0, r0, ah, nah, nal, f2_pk(V.x, V.y), f2_pk(V.z, V.w));
+            const float4 u = yr[b];
+            df_mac2(s0, r0, ah, nah, nal, f2_pk(u.x, u.z), f2_pk(u.y, u.w));
           }
         }
         const float2 S0 = f2_un(s0), R0 = f2_un(r0), S1 = f2_un(s1), R1 = f2_un(r1);
@@ -246,27 +249,30 @@ __global__ void __launch_bounds__(PD_THREADS, 3) k_pdig(SplitShared S, SplitWave
         if (gn > 1) Ps[K + kap] = make_float2(S0.y, R0.y);
         if (gn > 2) Ps[2 * K + kap] = make_float2(S1.x, R1.x);
         if (gn > 3) Ps[3 * K + kap] = make_float2(S1.y, R1.y);
+        mx[0] = max(mx[0], __float_as_uint(fabsf(S0.x)));
+        mx[1] = max(mx[1], __float_as_uint(fabsf(S0.y)));
+        mx[2] = max(mx[2], __float_as_uint(fabsf(S1.x)));
+        mx[3] = max(mx[3], __float_as_uint(fabsf(S1.y)));
       }
     }
-    __syncthreads();
-    // one exponent per row (G, g0 + gi) over its K values
-    for (int gi = warp; gi < gn; gi += PD_THREADS / 32) {
-      float m = 0.f;
-      for (int c = lane; c < K; c += 32) m = fmaxf(m, fabsf(Ps[gi * K + c].x));
-      for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      const int e = row_exponent(__double_as_longlong((double)m));
-      if (lane == 0) {
-        es[gi] = e;
-        eout[eg.aopre + g0 + gi] = (int16_t)max(-30000, e);
-      }
+    // one exponent per row (G, g0 + gi) over its K values (nonnegative floats
+    // order as their bit patterns)
+#pragma unroll
+    for (int gi = 0; gi < 4; ++gi) {
+      const unsigned m = __reduce_max_sync(0xffffffffu, mx[gi]);
+      if (lane == 0 && gi < gn) atomicMax(&pmax[gi], m);
     }
     __syncthreads();
+    if (g0 + gc < ng) stage(g0 + gc);
+    if (threadIdx.x < gn)
+      eout[eg.aopre + g0 + threadIdx.x] = (int16_t)max(
+          -30000, row_exponent(__double_as_longlong((double)__uint_as_float(pmax[threadIdx.x]))));
     // eight consecutive K of one row per thread: each digit plane gets one
     // 16-byte store (the eight are adjacent in the core-matrix tile)
     const int KT8 = KT / 8;
     for (int idx = threadIdx.x; idx < gn * KT8; idx += PD_THREADS) {
       const int gi = idx / KT8, c8 = (idx - gi * KT8) * 8;
-      const int e = es[gi];
+      const int e = row_exponent(__double_as_longlong((double)__uint_as_float(pmax[gi])));
       // scaled by 2^(6 - e) in two exact steps (|value| < 2^(e - 1)), digit s is a
       // multiple of 2^(-7 s): adding and taking away 1.5 2^(23 - 7 s) rounds to
       // it and leaves the exact rest (f32 only: the 64-bit conversions ran on the
