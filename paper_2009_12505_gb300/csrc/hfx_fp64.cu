@@ -326,8 +326,13 @@ __global__ void __launch_bounds__(kThreads) k_v3(ContractArgs A) {
 }
 
 // Sigma_FG -= sum_{al,a} C_AF[al][a][f] P_G[al][a][g]   for every F in M4(G).
+// The outputs (F, f, g) of all F are one list over the block's threads: F by F,
+// the 169 outputs of two 13-AO atoms left an eighth of the lanes idle and every
+// thread repeated each F's Sigma lookups.  Bound by the FP64 units: 72.5 ms F by
+// F on the 8-atom cell at cutoffs 12 / 16 / 12.
 __global__ void __launch_bounds__(kThreads) k_v4(ContractArgs A) {
-  __shared__ int flist[1024];
+  __shared__ int flist[1024], pre[1025];
+  __shared__ int64_t soff[1024], smoff[1024];
   __shared__ int nsel_s;
   const PairLoc L = locate(A, blockIdx.x, true);
   const WorkItem it = A.items[L.w];
@@ -343,28 +348,50 @@ __global__ void __launch_bounds__(kThreads) k_v4(ContractArgs A) {
   const double *P = A.scratch + A.p_off[L.w - A.w0] + eg.aopre;  // P[al][a][ncol]
   const int K = pA * na;
   const int nG0 = it.n[0] + eg.n[0], nG1 = it.n[1] + eg.n[1], nG2 = it.n[2] + eg.n[2];
-  unsigned long long macs = 0;
-  for (int k = 0; k < nsel; ++k) {
+  // Sigma offsets of each F's block and its mirror, and the outputs before it
+  for (int k = threadIdx.x; k < nsel; k += kThreads) {
     const NbrEntry ef = A.nbr[it.fbase + flist[k]];
-    const int nf = A.nao[ef.other];
-    const double *Caf = A.C.data + A.C.offs[ef.cblk];
-    const int nout = nf * ng;
-    const int64_t off = sig_offset(A, ef.other, eg.other, nG0 - ef.n[0], nG1 - ef.n[1],
-                                   nG2 - ef.n[2]);
-    const int64_t moff = (A.sym && it.role == 1)
-                             ? sig_offset(A, eg.other, ef.other, -(nG0 - ef.n[0]),
-                                          -(nG1 - ef.n[1]), -(nG2 - ef.n[2]))
-                             : -1;
-    for (int o = threadIdx.x; o < nout; o += kThreads) {
-      const int f = o / ng, g = o - f * ng;
-      double s = 0.0;
-      for (int r = 0; r < K; ++r) s = fma(Caf[(int64_t)r * nf + f], P[(int64_t)r * ncol + g], s);
-      if (off >= 0) fx_add(A.acc + 2 * (off + o), -s, A.err);
-      if (moff >= 0) fx_add(A.acc + 2 * (moff + g * nf + f), -s, A.err);
-    }
-    macs += (unsigned long long)nout * K;
+    soff[k] = sig_offset(A, ef.other, eg.other, nG0 - ef.n[0], nG1 - ef.n[1], nG2 - ef.n[2]);
+    smoff[k] = (A.sym && it.role == 1)
+                   ? sig_offset(A, eg.other, ef.other, -(nG0 - ef.n[0]), -(nG1 - ef.n[1]),
+                                -(nG2 - ef.n[2]))
+                   : -1;
+    pre[k + 1] = A.nao[ef.other] * ng;
   }
-  if (threadIdx.x == 0 && macs) atomicAdd(A.macs + 6, macs);
+  if (threadIdx.x == 0) pre[0] = 0;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    int sum = 0;
+    for (int k0 = 0; k0 < nsel; k0 += 32) {
+      const int k = k0 + threadIdx.x;
+      int v = k < nsel ? pre[k + 1] : 0;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, v, o);
+        if ((int)threadIdx.x >= o) v += u;
+      }
+      if (k < nsel) pre[k + 1] = sum + v;
+      sum += __shfl_sync(0xffffffffu, v, 31);
+    }
+  }
+  __syncthreads();
+  const int total = pre[nsel];
+  for (int o = threadIdx.x; o < total; o += kThreads) {
+    int lo = 0, hi = nsel - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (pre[mid] <= o) lo = mid; else hi = mid - 1;
+    }
+    const NbrEntry &ef = A.nbr[it.fbase + flist[lo]];
+    const int nf = A.nao[ef.other];
+    const int f = (o - pre[lo]) / ng, g = (o - pre[lo]) - f * ng;
+    const double *c = A.C.data + A.C.offs[ef.cblk] + f;
+    const double *q = P + g;
+    double s = 0.0;
+    for (int r = 0; r < K; ++r) s = fma(c[(int64_t)r * nf], q[(int64_t)r * ncol], s);
+    if (soff[lo] >= 0) fx_add(A.acc + 2 * (soff[lo] + (int64_t)f * ng + g), -s, A.err);
+    if (smoff[lo] >= 0) fx_add(A.acc + 2 * (smoff[lo] + (int64_t)g * nf + f), -s, A.err);
+  }
+  if (threadIdx.x == 0 && total) atomicAdd(A.macs + 6, (unsigned long long)total * K);
 }
 
 }  // namespace
