@@ -172,12 +172,12 @@ __global__ void __launch_bounds__(kThreads) k_adj_r(ContractArgs A) {
 }
 
 // dV_AB[al][be] = -1/2 sum over active G of sum_{b,g} C_BG[be][b][g] R[al][b][(G,g)],
-// one block per 32 al x 64 be of a pair: the product over (b, g) from shared
-// chunks of DV_K, 2 x 4 outputs a thread (six shared loads for eight
-// multiply-adds).  One block per pair with one output a thread read both
+// one block per 16 al x 64 be of a pair: the product over (b, g) from shared
+// chunks of DV_K, four outputs a thread (five shared loads for four
+// multiply-adds, which take thirteen times as long).  One block per pair with one output a thread read both
 // operands from global memory per multiply-add: 8.2 ms for what the FP64 units
 // do in 4.
-constexpr int DV_AL = 32, DV_BE = 64, DV_K = 32;
+constexpr int DV_AL = 16, DV_BE = 64, DV_K = 32;
 __global__ void __launch_bounds__(kThreads) k_adj_dv(ContractArgs A, int nta, int ntb) {
   __shared__ double Rs[DV_AL][DV_K + 1], Cs[DV_BE][DV_K + 1];
   const int64_t w = A.w0 + blockIdx.x / (nta * ntb);
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_dv(ContractArgs A, int nta, in
   const int ncol = A.ncol[it.b];
   const double *R = A.scratch + A.p_off[w - A.w0];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double s[2][4] = {{0.0, 0.0, 0.0, 0.0}, {0.0, 0.0, 0.0, 0.0}};
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
   for (int g_ = 0; g_ < it.nG; ++g_) {
     if (!(A.wg_flags[it.wg_off + g_] & 0xFu)) continue;
     const NbrEntry eg = A.nbr[it.gbase + g_];
@@ -207,13 +207,9 @@ __global__ void __launch_bounds__(kThreads) k_adj_dv(ContractArgs A, int nta, in
       __syncthreads();
       const int m = min(DV_K, n - k0);
       for (int q = 0; q < m; ++q) {
-        const double x0 = Rs[ty][q], x1 = Rs[ty + 16][q];
+        const double x0 = Rs[ty][q];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const double c = Cs[tx + 16 * j][q];
-          s[0][j] = fma(c, x0, s[0][j]);
-          s[1][j] = fma(c, x1, s[1][j]);
-        }
+        for (int j = 0; j < 4; ++j) s[j] = fma(Cs[tx + 16 * j][q], x0, s[j]);
       }
     }
   }
@@ -231,14 +227,12 @@ __global__ void __launch_bounds__(kThreads) k_adj_dv(ContractArgs A, int nta, in
   }
   double *out = A.dv + A.V.offs[it.vblk];
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int al = al0 + ty + 16 * i, be = be0 + tx + 16 * j;
-      if (al >= pA || be >= pB) continue;
-      out[(int64_t)al * pB + be] = -0.5 * s[i][j];
-      if (mir) mir[(int64_t)be * pA + al] = -0.5 * s[i][j];
-    }
+  for (int j = 0; j < 4; ++j) {
+    const int al = al0 + ty, be = be0 + tx + 16 * j;
+    if (al >= pA || be >= pB) continue;
+    out[(int64_t)al * pB + be] = -0.5 * s[j];
+    if (mir) mir[(int64_t)be * pA + al] = -0.5 * s[j];
+  }
 }
 
 // dC_BG[be][b][g] += -1/2 sum_al V_AB[al][be] R[al][b][(G,g)]   (C in the B
