@@ -463,46 +463,68 @@ __device__ __forceinline__ void zc_contract(const float2 (&z)[CW], int cend,
 // negatives and the negated low words, zero from column cend on (an odd last
 // pair repeats its column's Y, times zero).  Y words are loaded one by one
 // into the two lanes.  P1: so = 16, sc = 1; otherwise so = 1, sc = 16.
+// zc_outputs takes outputs o0 .. o0 + U - 1 over NJ column pairs.  NJ is a
+// constant and U small: with no branch between the pairs the compiler moves
+// their shared loads ahead, and it is the loads' latency, beside the MMAs'
+// operand reads, that bounds the contraction (half its arithmetic left its time
+// unchanged).  8-atom cell: 25.4 ms with a run-time number of pairs and groups
+// of four outputs, 23.7 with constants, 23.2 in groups of two (13 AOs; 16 AOs:
+// 13.3, 11.3 and 11.1 ms on a smaller cell; groups of five: 24.5).
+template <int NP, bool P1, int U, int NJ>
+__device__ __forceinline__ void zc_outputs(const uint64_t (&zh)[NP], const uint64_t (&nzh)[NP],
+                                           const uint64_t (&nzl)[NP], int cend,
+                                           const float *__restrict__ yf, int o0,
+                                           float2 *__restrict__ outp) {
+  constexpr int SO = P1 ? 32 : 2, SC = P1 ? 2 : 32;  // float words per output, column
+  uint64_t sh[U], sl[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) sh[u] = sl[u] = 0;
+#pragma unroll
+  for (int j = 0; j < NJ; ++j) {
+    // the pair's second column (only the last pair can lack one)
+    const int d1 = j + 1 < NJ || 2 * j + 1 < cend ? SC : 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const float *y = yf + (o0 + u) * SO + 2 * j * SC;
+      df_mac2(sh[u], sl[u], zh[j], nzh[j], nzl[j], f2_pk(y[0], y[d1]), f2_pk(y[1], y[d1 + 1]));
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const float2 h = f2_un(sh[u]), l = f2_un(sl[u]);
+    float th = h.x, tl = l.x;
+    df_add(th, tl, make_float2(h.y, l.y));
+    outp[(o0 + u) * 128] = make_float2(th, tl);
+  }
+}
+
+// Outputs 0 .. no - 1, two at a time.
+template <int NP, bool P1, int NJ>
+__device__ __forceinline__ void zc_contract_nj(const uint64_t (&zh)[NP], const uint64_t (&nzh)[NP],
+                                               const uint64_t (&nzl)[NP], int cend,
+                                               const float *__restrict__ yf, int no,
+                                               float2 *__restrict__ outp) {
+  int o = 0;
+  for (; o + 2 <= no; o += 2) zc_outputs<NP, P1, 2, NJ>(zh, nzh, nzl, cend, yf, o, outp);
+  for (; o < no; ++o) zc_outputs<NP, P1, 1, NJ>(zh, nzh, nzl, cend, yf, o, outp);
+}
+
 template <int NP, bool P1>
 __device__ __forceinline__ void zc_contract2(const uint64_t (&zh)[NP], const uint64_t (&nzh)[NP],
                                              const uint64_t (&nzl)[NP], int cend,
                                              const float2 *__restrict__ yb, int no,
                                              float2 *__restrict__ outp) {
   const float *yf = reinterpret_cast<const float *>(yb);
-  constexpr int SO = P1 ? 32 : 2, SC = P1 ? 2 : 32;  // float words per output, column
-  const int npair = (cend + 1) >> 1;
-  auto put = [&](int o, uint64_t h2, uint64_t l2) {
-    const float2 h = f2_un(h2), l = f2_un(l2);
-    float sh = h.x, sl = l.x;
-    df_add(sh, sl, make_float2(h.y, l.y));
-    outp[o * 128] = make_float2(sh, sl);
-  };
-  const int no4 = no & ~3;
-  for (int o0 = 0; o0 < no4; o0 += 4) {
-    uint64_t sh[4] = {0, 0, 0, 0}, sl[4] = {0, 0, 0, 0};
-#pragma unroll
-    for (int j = 0; j < NP; ++j) {
-      if (j >= npair) break;
-      const int d1 = 2 * j + 1 < cend ? SC : 0;  // the pair's second column
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float *y = yf + (o0 + u) * SO + 2 * j * SC;
-        df_mac2(sh[u], sl[u], zh[j], nzh[j], nzl[j], f2_pk(y[0], y[d1]), f2_pk(y[1], y[d1 + 1]));
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) put(o0 + u, sh[u], sl[u]);
-  }
-  for (int o = no4; o < no; ++o) {
-    uint64_t sh = 0, sl = 0;
-#pragma unroll
-    for (int j = 0; j < NP; ++j) {
-      if (j >= npair) break;
-      const int d1 = 2 * j + 1 < cend ? SC : 0;
-      const float *y = yf + o * SO + 2 * j * SC;
-      df_mac2(sh, sl, zh[j], nzh[j], nzl[j], f2_pk(y[0], y[d1]), f2_pk(y[1], y[d1 + 1]));
-    }
-    put(o, sh, sl);
+  // a copy for each number of column pairs: no branches between the pairs
+  switch ((cend + 1) >> 1) {
+    case 1: return zc_contract_nj<NP, P1, 1>(zh, nzh, nzl, cend, yf, no, outp);
+    case 2: return zc_contract_nj<NP, P1, 2>(zh, nzh, nzl, cend, yf, no, outp);
+    case 3: return zc_contract_nj<NP, P1, 3>(zh, nzh, nzl, cend, yf, no, outp);
+    case 4: return zc_contract_nj<NP, P1, 4>(zh, nzh, nzl, cend, yf, no, outp);
+    case 5: return zc_contract_nj<NP, P1, 5>(zh, nzh, nzl, cend, yf, no, outp);
+    case 6: return zc_contract_nj<NP, P1, 6>(zh, nzh, nzl, cend, yf, no, outp);
+    case 7: return zc_contract_nj<NP, P1, 7>(zh, nzh, nzl, cend, yf, no, outp);
+    default: return zc_contract_nj<NP, P1, 8>(zh, nzh, nzl, cend, yf, no, outp);
   }
 }
 
