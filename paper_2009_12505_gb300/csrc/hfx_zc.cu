@@ -47,9 +47,13 @@
 // k_zc takes the jobs whose blocks and atom A have at most 16 AOs, k_zcw
 // (hfx_zcw.cu) the others.  k_zcw's second tensor-core product was tried for
 // small blocks too: 31.7 ms with 8 epilogue warps and 34.3 ms with 16, against
-// 24.7 (8-atom cell).  There the operand stream (30 KB a stage, 24 B/clk per SM
-// from L2) and the MMAs' shared-memory reads already take 17 of the 19 thousand
-// cycles of a tile.
+// 24.7 (8-atom cell).
+//
+// What bounds k_zc: the contraction's shared-memory loads beside the MMAs'
+// operand reads.  In copies of the kernel on the 8-atom cell (25.7 ms), a quarter
+// of A's bytes changed nothing and no contraction at all took 18.3 ms; half the
+// contraction's arithmetic gained nothing either.  25.7 ms before the loader's lanes
+// and the contraction's unrolling, 23.2 ms now (8 ms of bf16 products).
 #include "zc_common.cuh"
 
 namespace split {

@@ -26,12 +26,14 @@
 // expiry the kernel records HFX_DEV_ERR_TIMEOUT, drains its copies and MMAs,
 // frees TMEM and returns.
 //
-// What bounds it: 22 operand stages a tile, which arrive at 24 B/clk per SM (the
-// whole chip's rate from L2), beside an epilogue of about 18 thousand cycles a
-// tile.  8-atom two-element cell (13/60 and 27/90, C, D to 9 bohr): 178.7 ms for
-// its wide jobs with the double-float contraction from global memory, 127 ms
-// with that contraction halved and Y staged, 113.9 ms now (35 ms of bf16
-// products at the sustained peak).
+// What bounds it: an epilogue of about 19 thousand cycles a tile, 5 thousand of
+// them waiting for the single Y buffer (five operand stages leave no room for a
+// second one; three stages and two buffers took 116 ms), beside up to 22 operand
+// stages.  8-atom two-element cell (13/60 and 27/90, C, D to 9 bohr): 178.7 ms
+// for its wide jobs with a double-float contraction from global memory, 127 ms
+// with that contraction halved and Y staged, 113.9 ms with this product, 109.7 ms
+// now, with one loader lane per stage (35 ms of bf16 products at the sustained
+// peak).
 #include "zc_common.cuh"
 
 namespace split {

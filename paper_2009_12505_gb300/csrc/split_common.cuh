@@ -37,19 +37,6 @@ __device__ __forceinline__ void to_digits(double x, int e, int (&d)[KS]) {
   d[0] = (int)X;
 }
 
-// k balanced base-128 digits of an integer X with |X| <= 2^(7 KS - 1):
-// X = sum_s d_s 2^(7 (KS - 1 - s)), |d_s| <= 64.
-template <int KS>
-__device__ __forceinline__ void to_digits_i64(long long X, int (&d)[KS]) {
-#pragma unroll
-  for (int s = KS - 1; s > 0; --s) {
-    const int dd = (int)(((X + 64) & 127) - 64);
-    d[s] = dd;
-    X = (X - dd) >> 7;
-  }
-  d[0] = (int)X;
-}
-
 // Add W * 2^e to a fixed-point Sigma element (hi: 2^-32 units, lo: 2^-64
 // units) with integer arithmetic; |W 2^e| < 2^31, else nothing is added and
 // HFX_DEV_ERR_BOUNDS is recorded in *err.
