@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(256) k_density(
   const int nK = nao[gr.K], nL = nao[gr.L];
   const int64_t aK = aoff[gr.K], aL = aoff[gr.L];
   const double inv = 1.0 / nk;
-  double mx = 0.0;
+  unsigned long long mx = 0;
   for (int t0 = 0; t0 < nK * nL; t0 += blockDim.x) {
     const int t = t0 + threadIdx.x;
     const bool live = t < nK * nL;
@@ -105,13 +105,14 @@ __global__ void __launch_bounds__(256) k_density(
       if (live && j < gr.count) {
         const DensityKey &e = dkeys[gr.first + j];
         out[e.off + (e.tr ? l * nK + k : t)] = re[j] * inv;
-        mx = fmax(mx, fabs(im[j] * inv));
+        mx = max(mx, (unsigned long long)__double_as_longlong(fabs(im[j] * inv)));
       }
     __syncthreads();
   }
-  for (int o = 16; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  // nonnegative doubles order as their bit patterns
-  if ((threadIdx.x & 31) == 0) atomicMax(maxim, (unsigned long long)__double_as_longlong(mx));
+  // nonnegative doubles order as their bit patterns, with NaN (an overflowed
+  // sum) above them all
+  for (int o = 16; o; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(maxim, mx);
 }
 
 constexpr int SK_KEYS = 256;  // keys whose phases are held at a time

@@ -36,6 +36,14 @@ def test_density_groups(nao, nbands, nk, reach):
     assert abs(maxim - np.abs(ref.imag).max()) <= tol
 
 
+def test_density_overflow_shows_in_max_imag():
+    """Finite coefficients whose products overflow: the imaginary part is no number, and says so."""
+    coef = np.full((1, 5, 2), 1e200 + 1e200j)
+    _, maxim = hfx.Context([2, 3], [4, 4]).density_from_eigvecs(
+        np.zeros((1, 3)), coef, np.ones((1, 2)), np.array([(0, 1, 0, 0, 0)]))
+    assert not np.isfinite(maxim)
+
+
 @pytest.mark.parametrize("nao", [2, 17])
 def test_sigma_k_many_keys(nao):
     s = synth.custom("one", 1.0, 1, [[0, 0, 0]], [nao], [2])
