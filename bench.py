@@ -116,8 +116,8 @@ def workload_desc(wl) -> str:
 # cell over its issued bf16 tensor flops, captured from the hfx_zc.cu whose code
 # (comments and blank space removed) has this sha256 prefix (see the k_zc
 # profile summary under profiles/)
-ZC_BYTES_PER_TENSOR_FLOP = (30.483057e9 + 0.469812e9) / 14.988985761792e12
-ZC_CAPTURED_SHA = "efee46cbd3e070ad"
+ZC_BYTES_PER_TENSOR_FLOP = (22.585361e9 + 0.377352e9) / 13.4e12
+ZC_CAPTURED_SHA = "b9c11dbd0960f869"
 
 
 def source_digest(path):
