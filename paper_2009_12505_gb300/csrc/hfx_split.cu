@@ -138,6 +138,83 @@ __global__ void k_slice_v(SplitShared S) {
   slice_row<KS>(src, grow, r, NT, pA, pB, S.ktY[it.b], S.vs + S.vs_base[e], S.vs_e);
 }
 
+// The last two bytes of x and y as one word, and bits 7 q .. 7 q + 6 of both
+// (q = 0, 1, from such a word) as bf16 of the field less 64: 0x4300 | v is 128 + v.
+__device__ __forceinline__ uint32_t pd_low16(int x, int y) {
+  return __byte_perm((uint32_t)x, (uint32_t)y, 0x5410);
+}
+__device__ __forceinline__ uint32_t pd_field(uint32_t v) {
+  v = (v & 0x007F007Fu) | 0x43004300u;
+  uint32_t d;
+  asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(v), "r"(0x43404340u));
+  return d;
+}
+// bf16 of two whole numbers of at most 2^8.
+__device__ __forceinline__ uint32_t pd_whole(int x, int y) {
+  uint32_t d;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;"
+      : "=r"(d)
+      : "f"(__int_as_float(0x4B400000 + y) - 12582912.f),
+        "f"(__int_as_float(0x4B400000 + x) - 12582912.f));
+  return d;
+}
+
+// Magnitude that a row's exponent comes from (bit pattern): the high word's, or 16
+// times the low word's where a cancelled sum left more than that in it.  So
+// |d_0| <= 64 + 4, and an order group's sum over K <= 640 stays exact in f32:
+// 640 64 (5 64 + 68) < 2^24.
+__device__ __forceinline__ uint32_t pd_mag(float h, float l) {
+  return __float_as_uint(fmaxf(fabsf(h), fabsf(16.f * l)));
+}
+
+// The KS balanced base-128 digits of two f32 pairs u and v in last units
+// 2^(e - 7 KS), as pairs of bf16.  The whole number X of a pair is the sum of its
+// two words, each rounded to the last unit (ties to even), and its digits are
+// those with -64 <= d_s <= 63 for s > 0 (X + 64 (1 + 128 + ..) has the plain
+// digits d_s + 64).  f1 f2 = 2^(7 KS - e - 21) in both lanes.  A word w is
+// split with f32 operations at 2^21 units: adding 1.5 2^23 leaves the nearest
+// whole number in the low mantissa bits, the rest times 2^21 is exact, and 2^21
+// being even the tie rule is that of w itself; 32-bit integer operations do the
+// rest (64-bit conversions ran on the FP64 pipe, at 1/64 of the rate).
+template <int KS>
+__device__ __forceinline__ void pd_digits(float2 u, float2 v, uint64_t f1, uint64_t f2,
+                                          uint32_t (&d)[KS]) {
+  const uint64_t M = f2_pk(12582912.f, 12582912.f), P = f2_pk(2097152.f, 2097152.f);
+  int hi[2], lo[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const float2 x = k ? v : u;
+    const uint64_t a = f2_mul(f2_mul(f2_pk(x.x, x.y), f1), f2);
+    const uint64_t w = f2_add(a, M);
+    const float2 h = f2_un(w), l = f2_un(f2_fma(f2_sub(a, f2_sub(w, M)), P, M));
+    hi[k] = (int)(__float_as_uint(h.x) + __float_as_uint(h.y) - 0x96800000u);
+    lo[k] = (int)(__float_as_uint(l.x) + __float_as_uint(l.y) - 0x96800000u);
+  }
+  if constexpr (KS > 3) {
+    constexpr int OL = 64 * (1 + 128 + 128 * 128);
+    constexpr int OH = KS == 6 ? 64 * (1 + 128) : KS == 5 ? 64 : 0;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      lo[k] += OL;
+      hi[k] += OH + (lo[k] >> 21);
+    }
+    const uint32_t l = pd_low16(lo[0], lo[1]);
+    d[KS - 1] = pd_field(l);
+    d[KS - 2] = pd_field(l >> 7);
+    d[KS - 3] = pd_field(pd_low16(lo[0] >> 14, lo[1] >> 14));
+    const uint32_t h = pd_low16(hi[0], hi[1]);
+    if constexpr (KS > 4) d[KS - 4] = pd_field(h);
+    if constexpr (KS > 5) d[KS - 5] = pd_field(h >> 7);
+    d[0] = pd_whole(hi[0] >> (7 * (KS - 4)), hi[1] >> (7 * (KS - 4)));
+  } else {
+    static_assert(KS == 2 || KS > 3);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) lo[k] += (hi[k] << 21) + 64;
+    d[1] = pd_field(pd_low16(lo[0], lo[1]));
+    d[0] = pd_whole(lo[0] >> 7, lo[1] >> 7);
+  }
+}
+
 // P of the D_AB piece, computed and sliced in one pass: one CTA per (pair, G)
 // of the wave's pairs with a D_AB job and D_AB survivors for G.
 //   P_G[(al,a)][g] = sum_b D_AB[a][b] Y[al][b][(G,g)]
@@ -221,7 +298,7 @@ __global__ void __launch_bounds__(PD_THREADS, 3) k_pdig(SplitShared S, SplitWave
         float sh = 0.f, sl = 0.f;
         for (int b = 0; b < nb; ++b) df_mac(sh, sl, d[b], y[b]);
         Ps[kap] = make_float2(sh, sl);
-        mx[0] = max(mx[0], __float_as_uint(fabsf(sh)));
+        mx[0] = max(mx[0], pd_mag(sh, sl));
       }
     } else {
       // all gn columns of one (al, a) per thread, two per packed (f32x2)
@@ -249,10 +326,10 @@ __global__ void __launch_bounds__(PD_THREADS, 3) k_pdig(SplitShared S, SplitWave
         if (gn > 1) Ps[K + kap] = make_float2(S0.y, R0.y);
         if (gn > 2) Ps[2 * K + kap] = make_float2(S1.x, R1.x);
         if (gn > 3) Ps[3 * K + kap] = make_float2(S1.y, R1.y);
-        mx[0] = max(mx[0], __float_as_uint(fabsf(S0.x)));
-        mx[1] = max(mx[1], __float_as_uint(fabsf(S0.y)));
-        mx[2] = max(mx[2], __float_as_uint(fabsf(S1.x)));
-        mx[3] = max(mx[3], __float_as_uint(fabsf(S1.y)));
+        mx[0] = max(mx[0], pd_mag(S0.x, R0.x));
+        mx[1] = max(mx[1], pd_mag(S0.y, R0.y));
+        mx[2] = max(mx[2], pd_mag(S1.x, R1.x));
+        mx[3] = max(mx[3], pd_mag(S1.y, R1.y));
       }
     }
     // one exponent per row (G, g0 + gi) over its K values (nonnegative floats
@@ -273,11 +350,9 @@ __global__ void __launch_bounds__(PD_THREADS, 3) k_pdig(SplitShared S, SplitWave
     for (int idx = threadIdx.x; idx < gn * KT8; idx += PD_THREADS) {
       const int gi = idx / KT8, c8 = (idx - gi * KT8) * 8;
       const int e = row_exponent(__double_as_longlong((double)__uint_as_float(pmax[gi])));
-      // scaled by 2^(6 - e) in two exact steps (|value| < 2^(e - 1)), digit s is a
-      // multiple of 2^(-7 s): adding and taking away 1.5 2^(23 - 7 s) rounds to
-      // it and leaves the exact rest (f32 only: the 64-bit conversions ran on the
-      // FP64 pipe).  Below 2^-200 the row is dropped.
-      const int sft = e > -200 ? 7 - e : 0, s1 = sft / 2, s2 = sft - s1;
+      // P 2^(7 KS - e - 21) in two exact steps: its whole part is the digits from
+      // 2^21 last units on.  Below 2^-200 the row is dropped.
+      const int sft = e > -200 ? 7 * KS - 21 - e : 0, s1 = sft / 2, s2 = sft - s1;
       const float q1 = e > -200 ? __int_as_float((s1 + 127) << 23) : 0.f;
       const float q2 = __int_as_float((s2 + 127) << 23);
       const uint64_t f1 = f2_pk(q1, q1), f2 = f2_pk(q2, q2);
@@ -286,23 +361,10 @@ __global__ void __launch_bounds__(PD_THREADS, 3) k_pdig(SplitShared S, SplitWave
       for (int k = 0; k < 4; ++k) {
         const int c = c8 + 2 * k;
         const float2 z = make_float2(0.f, 0.f);
-        const float2 u = c < K ? Ps[gi * K + c] : z, v = c + 1 < K ? Ps[gi * K + c + 1] : z;
-        // renormalised, so the low words are below the third digit
-        uint64_t h = 0, l = 0;
-        df_acc2(h, l, f2_mul(f2_mul(f2_pk(u.x, v.x), f1), f2));
-        df_acc2(h, l, f2_mul(f2_mul(f2_pk(u.y, v.y), f1), f2));
+        uint32_t d[KS];
+        pd_digits<KS>(c < K ? Ps[gi * K + c] : z, c + 1 < K ? Ps[gi * K + c + 1] : z, f1, f2, d);
 #pragma unroll
-        for (int sd = 0; sd < KS; ++sd) {
-          // digit as a whole number: 2^(7 sd) times the multiple
-          const float m = __int_as_float((23 - 7 * sd + 127) << 23 | 0x400000);
-          const float w = __int_as_float((7 * sd + 127) << 23);
-          const uint64_t M = f2_pk(m, m);
-          const uint64_t t = f2_sub(f2_add(h, M), M);
-          h = f2_sub(h, t);
-          if (sd == 2) h = f2_add(h, l);
-          const float2 d = f2_un(f2_mul(t, f2_pk(w, w)));
-          asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(pk[sd][k]) : "f"(d.y), "f"(d.x));
-        }
+        for (int sd = 0; sd < KS; ++sd) pk[sd][k] = d[sd];
       }
       const int r = eg.aopre + g0 + gi;
       const int rt = r / NT, rr = r - rt * NT, kt = c8 / TK, cc = c8 - kt * TK;
