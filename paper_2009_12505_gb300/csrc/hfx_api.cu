@@ -222,6 +222,7 @@ hfx_status fail(hfx_ctx *c, hfx_status s, const std::string &msg) {
   return s;
 }
 hfx_status fail_cuda(hfx_ctx *c, const char *what, cudaError_t e) {
+  cudaGetLastError();  // else the next call's first launch check reports it again
   return fail(c, HFX_E_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
