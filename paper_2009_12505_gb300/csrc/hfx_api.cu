@@ -69,8 +69,10 @@ struct Kind {
   std::unordered_map<uint64_t, Entry> map;
   std::vector<Chunk> chunks;
   std::vector<double> pending;
-  bool dirty = true;         // data or keys changed since the last pack
-  bool keys_changed = true;  // key set changed since the last plan
+  // changed since the last build that got as far as its screen: everything
+  // derived from the blocks is then known to be done, not only launched
+  bool dirty = true;         // data or keys
+  bool keys_changed = true;  // key set
   std::vector<uint64_t> keys;   // sorted, valid after pack
   std::vector<int64_t> offs;    // n + 1
   DevBuf<double> data;
@@ -279,6 +281,7 @@ void build_table(const std::vector<uint64_t> &keys, const std::vector<int64_t> &
 }
 
 // Pack one kind into a key-sorted device array and compute block upper limits.
+// Can be repeated: the caller clears K.dirty once the work launched here is done.
 hfx_status pack_kind(hfx_ctx *ctx, int k) {
   Kind &K = ctx->K[k];
   if (!K.dirty) return HFX_OK;
@@ -396,11 +399,11 @@ hfx_status pack_kind(hfx_ctx *ctx, int k) {
   CK(K.maxabs.reserve(nblk + 1));
   CK(launch_maxabs(K.data.p, K.d_offs.p, nblk, K.maxabs.p, ctx->d_err.p, st));
   ctx->launches += nblk > 0;
-  K.dirty = false;
   return HFX_OK;
 }
 
-// Neighbour lists and work items from the C and V key sets; D lookups.
+// Neighbour lists and work items from the C and V key sets; D lookups.  The
+// caller clears the change flags once the copies made here are done.
 hfx_status build_plan(hfx_ctx *ctx) {
   Kind &C = ctx->K[0], &V = ctx->K[1], &D = ctx->K[2];
   cudaStream_t st = ctx->stream;
@@ -509,8 +512,6 @@ hfx_status build_plan(hfx_ctx *ctx) {
       CK(cudaMemcpyAsync(ctx->d_items.p, ctx->items.data(), sizeof(WorkItem) * ctx->items.size(),
                          cudaMemcpyHostToDevice, st));
   }
-  C.keys_changed = V.keys_changed = D.keys_changed = false;
-  ctx->plan_valid = true;
   return HFX_OK;
 }
 
@@ -1095,10 +1096,8 @@ hfx_status hfx_build(hfx_ctx *ctx, double theta, hfx_prec prec, int32_t nslices,
     unsigned perr = 0;
     CK(cudaMemcpyAsync(&perr, ctx->d_err.p, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    if (perr & HFX_DEV_ERR_NONFINITE) {
-      for (int k = 0; k < 3; ++k) ctx->K[k].dirty = true;  // re-check on the next build
+    if (perr & HFX_DEV_ERR_NONFINITE)
       return fail(ctx, HFX_E_ARG, "non-finite value in an input block");
-    }
     hfx_status s = build_plan(ctx);
     if (s != HFX_OK) return s;
   }
@@ -1163,6 +1162,13 @@ hfx_status hfx_build(hfx_ctx *ctx, double theta, hfx_prec prec, int32_t nslices,
     kms[0] = ms;
     break;
   }
+  // The screen has run on the packed blocks, their upper limits, the mirror
+  // answer and the plan, so all of them are done.  A build that fails before
+  // this point leaves the flags standing and the next one does it all again: a
+  // row of the screen ends at the first word of F that all fall, so a neighbour
+  // order older than the upper limits would lose terms.
+  for (int k = 0; k < 3; ++k) ctx->K[k].dirty = ctx->K[k].keys_changed = false;
+  ctx->plan_valid = true;
   // ---- Sigma key set: collect, sort, offsets, lookup table
   const int64_t nsig = (int64_t)counters[7];
   {
@@ -1600,11 +1606,7 @@ namespace {
 // Copy one kind of a cell's blocks into the merged system m, atoms offset
 // by first (blocks already there are replaced).
 hfx_status copy_cell_kind(hfx_ctx *m, hfx_ctx *ctx, int k, int32_t first) {
-  // packing here must not hide from the cell's own next build that its
-  // blocks changed since its last one: keep the kind's dirty flag
-  const bool was_dirty = ctx->K[k].dirty;
   hfx_status s = pack_kind(ctx, k);
-  ctx->K[k].dirty = was_dirty;
   if (s != HFX_OK) return s;
   if (ctx->stream && cudaStreamSynchronize(ctx->stream) != cudaSuccess)
     return fail(ctx, HFX_E_CUDA, "batch: stream synchronisation failed");

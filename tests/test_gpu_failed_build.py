@@ -67,3 +67,15 @@ def test_failure_is_reported_once(workloads, mode):
     ctx.build(THETA, *mode)
     _failing_build(ctx, stream, *mode)
     _same_as_fresh(workloads[0], ctx, *mode)
+
+
+@pytest.mark.parametrize("mode", [("fp64", 0), ("ozaki", 6)])
+def test_repeat_after_new_values(workloads, mode):
+    """C got new values before the failed build.  The screen ends a row at the first 32 neighbours that
+    all fall, so with an order or upper limits older than the values it would lose terms."""
+    a, b = workloads
+    ctx, stream = _context(a)
+    ctx.build(THETA, *mode)
+    ctx.set_blocks("C", b.C)
+    _failing_build(ctx, stream, *mode)
+    _same_as_fresh(b, ctx, *mode)
