@@ -160,7 +160,7 @@ struct hfx_ctx {
   DevBuf<int64_t> d_waveoffs;
 
   // split-precision (HFX_OZAKI) operands
-  int split_ks = 0;
+  int split_ks = 0;  // digits of C and V as they are now (0: not sliced since they changed)
   DevBuf<__nv_bfloat16> d_cy, d_c4, d_vs, d_ps, d_cz;
   DevBuf<int16_t> d_cy_e, d_c4_e, d_vs_e, d_ps_e, d_cz_e;
   DevBuf<int64_t> d_cz_meta;      // cz_base, cz_rowpre, czw_base, czw_rowpre
@@ -254,6 +254,7 @@ void invalidate(hfx_ctx *ctx, int k, bool keys) {
   ++ctx->gen[k];
   if (keys) ++ctx->kgen[k];
   if (k < 2) ctx->eri_valid = false;
+  if (k < 2) ctx->split_ks = 0;
   if (keys) ctx->K[k].keys_changed = true;
   if (keys && k == 2) ctx->dz_nd = -1;
   ctx->results_valid = false;
@@ -668,7 +669,6 @@ hfx_status split_prepare(hfx_ctx *ctx, int ks) {
   CK(cudaMemcpyAsync(ctx->d_kt.p, kt.data(), sizeof(int32_t) * kt.size(), cudaMemcpyHostToDevice,
                      st));
   CK(cudaStreamSynchronize(st));
-  ctx->split_ks = ks;
   return HFX_OK;
 }
 
@@ -1078,7 +1078,6 @@ hfx_status hfx_build(hfx_ctx *ctx, double theta, hfx_prec prec, int32_t nslices,
   CK(cudaEventRecord(ctx->ev[0], st));
   CK(cudaMemsetAsync(ctx->d_err.p, 0, sizeof(unsigned), st));
   const bool vd_dirty = ctx->K[1].dirty || ctx->K[2].dirty;
-  const bool cv_dirty = ctx->K[0].dirty || ctx->K[1].dirty || !ctx->plan_valid;
   ctx->c_reordered = ctx->K[0].dirty;
   for (int k = 0; k < 3; ++k) {
     hfx_status s = pack_kind(ctx, k);
@@ -1213,7 +1212,8 @@ hfx_status hfx_build(hfx_ctx *ctx, double theta, hfx_prec prec, int32_t nslices,
   }
   SplitShared SS{};
   if (split) {
-    if (cv_dirty || ctx->split_ks != nslices) {
+    if (ctx->split_ks != nslices) {
+      ctx->split_ks = 0;  // until this build has run on them
       hfx_status s = split_prepare(ctx, nslices);
       if (s != HFX_OK) return s;
       SS = split_shared(ctx);
@@ -1223,6 +1223,7 @@ hfx_status hfx_build(hfx_ctx *ctx, double theta, hfx_prec prec, int32_t nslices,
                        (SS.h_cz_rows > 0) + (SS.h_czw_rows > 0);
     }
     if (ctx->dz_nd < 0 || ctx->dz_ks != nslices) {
+      ctx->dz_nd = -1;
       hfx_status s = dz_prepare_meta(ctx, nslices);
       if (s != HFX_OK) return s;
     }
@@ -1540,6 +1541,7 @@ hfx_status hfx_build(hfx_ctx *ctx, double theta, hfx_prec prec, int32_t nslices,
   CK(cudaMemcpyAsync(kmacs, ctx->d_counters.p + 8, sizeof(kmacs), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   if (herr) return fail(ctx, HFX_E_CUDA, "contraction kernels reported error " + std::to_string(herr));
+  if (split) ctx->split_ks = nslices;
   float ms01 = 0, ms12 = 0, ms23 = 0, ms03 = 0;
   cudaEventElapsedTime(&ms01, ctx->ev[0], ctx->ev[1]);
   cudaEventElapsedTime(&ms12, ctx->ev[1], ctx->ev[2]);

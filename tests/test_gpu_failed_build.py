@@ -1,4 +1,4 @@
-"""Builds that fail on the host and are repeated.
+"""Builds that fail on the host and are repeated, and builds of different modes in turn.
 
 The failure is a build on a stream that is being captured: its work is recorded, not run, and its first
 wait is an error."""
@@ -79,3 +79,14 @@ def test_repeat_after_new_values(workloads, mode):
     ctx.set_blocks("C", b.C)
     _failing_build(ctx, stream, *mode)
     _same_as_fresh(b, ctx, *mode)
+
+
+@pytest.mark.parametrize("nslices", [4, 6])
+def test_split_after_fp64(workloads, nslices):
+    """C got new values and an FP64 build before the split build of the same digit count."""
+    a, b = workloads
+    ctx, _ = _context(a)
+    ctx.build(THETA, "ozaki", nslices)
+    ctx.set_blocks("C", b.C)
+    ctx.build(THETA, "fp64")
+    _same_as_fresh(b, ctx, "ozaki", nslices)
