@@ -616,76 +616,8 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
 
   if (warp == ZC_EPI) {
     // ------------------------------------------------------------ A / B loader
-    // the whole warp walks the steps.  Lane l holds entry q0 + l of the job
-    // (fetched 32 at a time, off the per-stage path) and waits for its stage,
-    // arms it and issues its copies itself, so a stage costs no shuffles; the
-    // lanes take turns, as the ring's parities need the stages in order
-    int s = 0;           // the ring's slot and the parity of its last release
-    uint32_t ph = 1;     // (the first round waits for none)
-    int step = 0, last = -1;  // stages passed, the last one this lane armed
-    bool ok = true;
-    for (int p = 0; p < npair && ok; ++p) {
-      // one decision for the whole warp
-      if (__shfl_sync(0xffffffffu, lane == 0 ? *abort_f : 0, 0)) break;
-      ZcPair<PAIR> pr;
-      pr.begin(p, ncj);
-      ZcLd L, Lo;  // L: the job of the current tile, Lo: the pair's other job
-      zc_ld_job<false>(S, W, cfg.jbeg, pr.r0, L);
-      pr.m0 = L.mtz;
-      if (pr.two) {
-        zc_ld_job<false>(S, W, cfg.jbeg, pr.r1, Lo);
-        pr.m1 = Lo.mtz;
-      }
-      int cur = 0, x, mt;
-      while (ok && pr.next(x, mt)) {
-        if (x != cur) {
-          zc_swap(L, Lo);
-          cur = x;
-        }
-        const uint32_t bb = (uint32_t)(KS * 16 * 2) * (uint32_t)L.Rl;  // bytes of a B block
-        for (int q0 = 0; q0 < L.nent && ok; q0 += 32) {
-          if (L.held != q0) {
-            if (q0 + lane < L.nent) L.mine = W.zc_ents[L.ent + q0 + lane];
-            L.held = q0;
-          }
-          const int nq = min(32, L.nent - q0);
-          const __nv_bfloat16 *a = L.A + ((int64_t)mt * L.ktot + L.mine.kofs) * KS * 128;
-          const __nv_bfloat16 *b0 = L.mine.dz[0] >= 0 ? S.dz + L.mine.dz[0] : S.dzero;
-          const __nv_bfloat16 *b1 = L.mine.dz[1] >= 0 ? S.dz + L.mine.dz[1] : S.dzero;
-          for (int qq = 0; qq < nq; ++qq) {
-            if (lane == qq) {
-              // once the build is given up, a stage that is not free stays so
-              ok = step < NST || umma::mbar_try_wait(&ctl->empty[s], ph) ||
-                   (!*abort_f && umma::mbar_wait(&ctl->empty[s], ph, S.err, ZC_WAIT));
-              if (!ok) {
-                *abort_f = 1;
-              } else {
-                last = step;
-                uint8_t *st = smem + s * STG;
-                umma::mbar_arrive_expect_tx(&ctl->full[s], A_BYTES + bb * (uint32_t)L.nblk);
-                umma::bulk_g2s(st, a, A_BYTES, &ctl->full[s]);
-                // B stage block-major: block b's KS digits of Rl rows x 16 K at b KS 16 16
-                umma::bulk_g2s(st + A_BYTES, b0, bb, &ctl->full[s]);
-                if (L.nblk > 1)
-                  umma::bulk_g2s(st + A_BYTES + KS * 16 * 16 * 2, b1, bb, &ctl->full[s]);
-              }
-            }
-            __syncwarp();
-            ++step;
-            if (++s == NST) {
-              s = 0;
-              ph ^= 1;
-            }
-          }
-          ok = __all_sync(0xffffffffu, ok);
-        }
-      }
-    }
-    // drain: the last stages issued must have landed before the CTA exits
-    last = __reduce_max_sync(0xffffffffu, last);
-    if (lane == 0)
-      for (int t = max(0, last + 1 - NST); t <= last; ++t)
-        umma::mbar_wait(&ctl->full[t % NST], (uint32_t)((t / NST) & 1), S.err, ZC_WAIT);
+    zc_loader<KS, NST, false, PAIR>(S, W, cfg.jbeg, ncj, npair, smem, ctl->full, ctl->empty,
+                                    abort_f, lane);
   } else if (warp == ZC_EPI + 2) {
     // ------------------------------------------------------------ Y loader
     if constexpr (YST) {
@@ -738,6 +670,10 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
           }
         }
       }
+      // copies of tiles that nobody waits for any more after a failure elsewhere
+      if (lane == 0)
+        for (long long t = max(0ll, hand - 2); t < hand; ++t)
+          umma::mbar_wait(&ctl->yfull[t & 1], (uint32_t)((t >> 1) & 1), S.err, ZC_WAIT);
     }
   } else if (warp == ZC_EPI + 1) {
     // ------------------------------------------------------------ MMA issuer

@@ -8,6 +8,7 @@
 
 #include "hfx_split.h"
 #include "split_common.cuh"
+#include "stage_ring.h"
 
 namespace split {
 
@@ -244,6 +245,74 @@ __device__ __forceinline__ void zc_ld_job(const SplitShared &S, const SplitWave 
                : (S.nabf[it.a] * S.nao[it.a] + 127) / 128;
   L.held = -1;
   L.mine = ZcEnt{0, {-1, -1}};
+}
+
+// The A / B loader of both kernels, by one whole warp: the jobs' operand stages
+// into the ring of NST stages at smem.  Lane l holds entry q0 + l of the job
+// (fetched 32 at a time, off the per-stage path) and waits for its stage, arms
+// it and issues its copies itself; the lanes take turns, as the ring's parities
+// need the stages in order, and one vote a stage ends the walk in all of them.
+template <int KS, int NST, bool WIDE, bool PAIR>
+__device__ __forceinline__ void zc_loader(const SplitShared &S, const SplitWave &W, int jbeg,
+                                          int ncj, int npair, uint8_t *smem, uint64_t *full,
+                                          uint64_t *empty, volatile int *abort_f, int lane) {
+  constexpr int A_BYTES = KS * 128 * 16 * 2;
+  constexpr int STG = A_BYTES + KS * ZC_COLS * 16 * 2;
+  StageRing<NST> ring;
+  bool ok = true;
+  for (int p = 0; p < npair && ok; ++p) {
+    // one decision for the whole warp
+    if (__shfl_sync(0xffffffffu, lane == 0 ? *abort_f : 0, 0)) break;
+    ZcPair<PAIR> pr;
+    pr.begin(p, ncj);
+    ZcLd L, Lo;  // L: the job of the current tile, Lo: the pair's other job
+    zc_ld_job<WIDE>(S, W, jbeg, pr.r0, L);
+    pr.m0 = L.mtz;
+    if (pr.two) {
+      zc_ld_job<WIDE>(S, W, jbeg, pr.r1, Lo);
+      pr.m1 = Lo.mtz;
+    }
+    int cur = 0, x, mt;
+    while (ok && pr.next(x, mt)) {
+      if (x != cur) {
+        zc_swap(L, Lo);
+        cur = x;
+      }
+      const uint32_t bb = (uint32_t)(KS * 16 * 2) * (uint32_t)L.Rl;  // bytes of a B block
+      for (int q0 = 0; q0 < L.nent && ok; q0 += 32) {
+        if (L.held != q0) {
+          if (q0 + lane < L.nent) L.mine = W.zc_ents[L.ent + q0 + lane];
+          L.held = q0;
+        }
+        const __nv_bfloat16 *a = L.A + ((int64_t)mt * L.ktot + L.mine.kofs) * KS * 128;
+        const __nv_bfloat16 *b0 = L.mine.dz[0] >= 0 ? S.dz + L.mine.dz[0] : S.dzero;
+        const __nv_bfloat16 *b1 = L.mine.dz[1] >= 0 ? S.dz + L.mine.dz[1] : S.dzero;
+        ok = ring_stages(
+            ring, min(32, L.nent - q0),
+            [&](int q) {
+              if (lane != q) return true;
+              if (!ring.fresh() && !umma::mbar_try_wait(&empty[ring.s], ring.ph) &&
+                  (*abort_f || !umma::mbar_wait(&empty[ring.s], ring.ph, S.err, ZC_WAIT))) {
+                *abort_f = 1;
+                return false;
+              }
+              uint8_t *st = smem + ring.s * STG;
+              uint64_t *bar = &full[ring.s];
+              umma::mbar_arrive_expect_tx(bar, A_BYTES + bb * (uint32_t)L.nblk);
+              umma::bulk_g2s(st, a, A_BYTES, bar);
+              // B stage block-major: block b's KS digits of Rl rows x 16 K at b KS 16 16
+              umma::bulk_g2s(st + A_BYTES, b0, bb, bar);
+              if (L.nblk > 1) umma::bulk_g2s(st + A_BYTES + KS * 16 * 16 * 2, b1, bb, bar);
+              return true;
+            },
+            [](bool c) { return __all_sync(0xffffffffu, c) != 0; });
+      }
+    }
+  }
+  // the last stages armed must have landed before the CTA exits
+  if (lane == 0)
+    for (int t = ring.pending(); t < ring.step; ++t)
+      umma::mbar_wait(&full[t % NST], (uint32_t)((t / NST) & 1), S.err, ZC_WAIT);
 }
 
 }  // namespace split
