@@ -341,9 +341,13 @@ __global__ void __launch_bounds__(PD_THREADS, 3) k_pdig(SplitShared S, SplitWave
     }
     __syncthreads();
     if (g0 + gc < ng) stage(g0 + gc);
-    if (threadIdx.x < gn)
-      eout[eg.aopre + g0 + threadIdx.x] = (int16_t)max(
-          -30000, row_exponent(__double_as_longlong((double)__uint_as_float(pmax[threadIdx.x]))));
+    if (threadIdx.x < gn) {
+      const float m = __uint_as_float(pmax[threadIdx.x]);
+      eout[eg.aopre + g0 + threadIdx.x] =
+          (int16_t)max(-30000, row_exponent(__double_as_longlong((double)m)));
+      // P (or its Y) beyond the f32 range has no digits: the build fails
+      if (!(m < INFINITY)) atomicOr(S.err, HFX_DEV_ERR_BOUNDS);
+    }
     // eight consecutive K of one row per thread: each digit plane gets one
     // 16-byte store (the eight are adjacent in the core-matrix tile)
     const int KT8 = KT / 8;

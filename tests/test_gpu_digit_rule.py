@@ -13,12 +13,12 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-def _sigma(k, y0, c, d):
+def _sigma(k, y0, c, d, y1=1.0):
     z = (0, 0, 0)
     ctx = hfx.Context([1, 1, 1, 1], [2, 1, 1, 1])
     ctx.set_block("C", 0, 2, z, [0.0, c])
     ctx.set_block("C", 1, 3, z, [1.0])
-    ctx.set_block("V", 0, 1, z, [y0, 1.0])
+    ctx.set_block("V", 0, 1, z, [y0, y1])
     ctx.set_block("D", 0, 1, z, [d])
     ctx.build(0.0, *(("bf16x3", 2) if k == 2 else ("ozaki", k)))
     assert ctx.keys().tolist() == [[2, 3, 0, 0, 0]]
@@ -45,3 +45,15 @@ def test_digit_range(k):
         pytest.skip("no CUDA device")
     u = 2.0 ** (2 - 7 * k)
     assert _sigma(k, 2.0 ** (7 * k - 8), 1.0 + 2.0 ** -12, 64.0 * u) == -(64.0 + 128.0 * 2.0 ** -12) * u
+
+
+@pytest.mark.parametrize("k", [4, 5, 6])
+@pytest.mark.parametrize("y0,y1,c,d", [(1e30, 1e30, 1e-55, 1e30), (1e30, 1.0, 1e-28, 1e30),
+                                       (1e39, 1e39, 1e-38, 1.0), (-1e30, 1.0, 1e-28, 1e30)])
+def test_overflow_fails(k, y0, y1, c, d):
+    """P beyond the f32 range (its own row's or another, from D Y or already in Y): an error, not a Sigma
+    without the row."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    with pytest.raises(hfx.HfxError):
+        _sigma(k, y0, c, d, y1)
