@@ -766,7 +766,8 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
         if (hf == 0 && (q4 == 0 || pr.two))
           zc_epi_job<false>(S, W, cfg.jbeg, q4 ? pr.r1 : pr.r0, lane, ctl->ej[pp][q4]);
       } else if (q4 == 2 || pr.two) {
-        zc_epi_ecol<ZC_CW>(S, W, cfg.jbeg, q4 == 3 ? pr.r1 : pr.r0, hf, lane, ctl->ecol[q4 - 2]);
+        const int e = zc_col_exp<ZC_CW>(S, W, cfg.jbeg, q4 == 3 ? pr.r1 : pr.r0, hf, lane);
+        if (lane < ZC_CW) ctl->ecol[q4 - 2][hf * ZC_CW + lane] = e;
       }
       asm volatile("bar.sync 1, %0;" ::"r"(ZC_ET) : "memory");
       pr.m0 = ctl->ej[pp][0].mtz;

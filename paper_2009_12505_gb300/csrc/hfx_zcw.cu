@@ -12,78 +12,81 @@
 //  * tcgen05.ld 16x256b gives a warp a 16 x 16 piece of Z in the fragment layout
 //    of mma.sync's A operand; each epilogue warp takes one such piece (its rows
 //    and column group) and no data moves between warps until the job ends;
-//  * Z and Y become six digits of 8 bits (exact in bf16).  Y of one al has its
-//    own exponent, Z takes the rest of the job's scale 2^E, which follows the
-//    largest product seen, so al of very different norm lose nothing; digit
-//    products of one order are exact in f32, and the orders join double-float
-//    sums.  The digits end 2^-48 below the largest product, the digits of the
-//    first product 2^-42 below their rows, so the error of Sigma is the latter's.
+//  * Z and Y become six digits of 8 bits (exact in bf16), Z with an exponent per
+//    row of the fragment, Y with one per (al, output); D's column exponents, which
+//    Z's columns are in units of, are multiplied into Y.  Digit products of one
+//    order are exact in f32; the orders, scaled by both exponents, join the
+//    double-float sum of their (row, output).
+// Precision: the digits drop what is 2^-48 below the largest Z of the row times the
+// largest Y of that al and output (over at most 16 columns, each in units of its
+// D column).  The first product has already rounded every Z to 2^-42 of its C row
+// times its D column, so each element of Sigma, small or large, has the error of
+// the first product alone.  (One exponent per al and a scale per job, relative to
+// the largest product of all, left outputs 2^-24 below the largest with 24 bits.)
 //
 // Roles (one CTA per SM, persistent): warps 0-15 as above; warp 16 streams A and
 // B tiles into a ring of shared stages, warp 17 issues the tcgen05 MMAs into one
-// of two TMEM accumulators, warp 18 copies each tile's Y rows and row exponents,
-// warps 18 and 19 find the exponent of each al's Y.  Every wait is bounded; on
-// expiry the kernel records HFX_DEV_ERR_TIMEOUT, drains its copies and MMAs,
+// of two TMEM accumulators, warp 18 copies each tile's Y rows and row
+// exponents.  Every wait is bounded; on expiry the kernel records HFX_DEV_ERR_TIMEOUT, drains its copies and MMAs,
 // frees TMEM and returns.
 //
-// What bounds it: an epilogue of about 19 thousand cycles a tile, 5 thousand of
-// them waiting for the single Y buffer (five operand stages leave no room for a
-// second one; three stages and two buffers took 116 ms), beside up to 22 operand
-// stages.  8-atom two-element cell (13/60 and 27/90, C, D to 9 bohr): 178.7 ms
-// for its wide jobs with a double-float contraction from global memory, 127 ms
-// with that contraction halved and Y staged, 113.9 ms with this product, 109.7 ms
-// now, with one loader lane per stage (35 ms of bf16 products at the sustained
-// peak).
+// What bounds it: the epilogue, beside up to 22 operand stages a tile; it also
+// waits for the single Y buffer (five operand stages leave no room for a second
+// one; three stages and two buffers took 116 ms where this took 109.7).  8-atom
+// two-element cell (13/60 and 27/90, C, D to 9 bohr): 178.7 ms for its wide jobs
+// with a double-float contraction from global memory, 127 ms with that contraction
+// halved and Y staged, 109.7 ms with this product and two warps that looked for
+// one exponent per al before a tile could be read; with the exponents taken from
+// each fragment's own loads the whole step went from 144.5 to 134.5 ms (35 ms of
+// bf16 products at the sustained peak in this kernel).
 #include "zc_common.cuh"
 
 namespace split {
 
 // Epilogue: 16 warps, one per TMEM lane quarter, group of 16 columns and 16-row
-// fragment, so that each scheduler has four of them to hide latencies; 20
-// warps in all leave 96 registers a thread.
+// fragment, so that each scheduler has four of them to hide latencies; with the
+// other roles a scheduler has five warps, which leaves 96 registers a thread.
 constexpr int ZC_EPI = 16;
 constexpr int ZC_NQ = 2;                         // column groups
 constexpr int ZC_CW = ZC_COLS / ZC_NQ;           // Z columns per epilogue warp
 constexpr int ZC_ET = ZC_EPI * 32;               // epilogue threads
-constexpr int ZC_THREADS = (ZC_EPI + 4) * 32;    // + A/B loader, MMA issuer, two Y warps
-// Staged Y rows of one al end with a pad of ZC_YPAD pairs, which holds the
-// exponent of the al's Y and moves the rows of the next al to other banks.
+constexpr int ZC_THREADS = (ZC_EPI + 3) * 32;    // + A/B loader, MMA issuer, Y loader
+// Staged Y rows of one al end with a pad of ZC_YPAD pairs, which moves the rows
+// of the next al to other banks.
 constexpr int ZC_YPAD = 2;
 constexpr int ZC_PASS = 8;   // outputs of a block per pass through the reduction buffer
 constexpr int ZC_DIG = 6;    // digits of the second product's operands (8 bits each)
-constexpr int ZC_NOEXP = -1000;
 
 struct ZcwSmem {
-  uint64_t full[8], empty[8], tfull[2], tempty[2], yfull[2], yrdy[2], yempty[2], drain;
+  uint64_t full[8], empty[8], tfull[2], tempty[2], yfull[2], yempty[2], drain;
   unsigned long long t_start;  // globaltimer at the start of the roles
   uint32_t tslot;
   int abort_f;
   __align__(16) int16_t erow[2][128];  // row exponents of the tile in each Y buffer
-  int ecol[2][ZC_COLS];  // column exponents of the pair's jobs (column group q at q * CW)
+  // column exponents of the pair's jobs: the largest of each column group, and
+  // each column's 2^(exponent - largest) (column group q at q * CW)
+  int emax[2][ZC_NQ];
+  __align__(8) float cw[2][ZC_COLS];
   ZcEpiJob ej[2][2];     // [pair parity][job of the pair]
 };
 
-// Exponent e of one al's Y for one block of a tile, by one warp: every |Y| <
-// 2^e over all b and g (-128: all zero, or below 2^-120).  y: the al's [b][16]
-// pairs of 16-column block 0, kstr pairs to the next block.
-__device__ __forceinline__ int zc_y_exp(const float2 *y, int64_t kstr, int nb, int ng, int lane) {
-  unsigned m = 0;
-  for (int k = 0; 16 * k < ng; ++k) {
-    const float4 *r = reinterpret_cast<const float4 *>(y + k * kstr);
-    const int g = 2 * (lane & 7), n = ng - 16 * k;
-    for (int i = lane; i < nb * 8; i += 32) {
-      const float4 v = r[i];  // pairs (b, g), (b, g + 1)
-      if (g < n) m = max(m, __float_as_uint(fabsf(v.x)));
-      if (g + 1 < n) m = max(m, __float_as_uint(fabsf(v.z)));
-    }
-  }
-  const int e = (int)(__reduce_max_sync(0xffffffffu, m) >> 23) - 126;
-  return e < -120 ? -128 : min(e, 126);
+// 2^e as f32: zero below the normal range, 2^127 above it (both are far outside
+// what Sigma's words hold, |x| from 2^-64 to 2^31).
+__device__ __forceinline__ float zc_exp2(int e) {
+  return e < -126 ? 0.f : __int_as_float((min(e, 127) + 127) << 23);
 }
 
-// 2^e as f32, zero below the normal range (e <= 127).
-__device__ __forceinline__ float zc_exp2(int e) {
-  return e < -126 ? 0.f : __int_as_float((e + 127) << 23);
+// From the largest magnitude's bit pattern: e with |x| < 2^e, and 2^-e (NaN from
+// 2^126 on, infinities and NaN included: the sums carry it to the range check).
+__device__ __forceinline__ int zc_exp_of(uint32_t m, float &sc) {
+  const int f = (int)(m >> 23);
+  sc = f > 252 ? __int_as_float(0x7FC00000) : __int_as_float((253 - f) << 23);
+  return f - 126;
+}
+
+__device__ __forceinline__ uint32_t zc_max_abs(uint64_t v) {
+  const float2 x = f2_un(v);
+  return max(__float_as_uint(fabsf(x.x)), __float_as_uint(fabsf(x.y)));
 }
 
 __device__ __forceinline__ void zc_mma(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2,
@@ -112,22 +115,24 @@ __device__ __forceinline__ uint32_t zc_digit(int i, uint64_t &h, uint64_t l) {
 }
 
 // This lane's part of the 16 x 8 fragment of Y (contracted index k .. = kc +
-// {0, 1, 8, 9}, one output): pairs y[k] (P1) or y[16 k], times sc, as f32x2 of
-// the high and of the low words.  nk: valid k; live: it is an output.
+// {0, 1, 8, 9}, one output): pairs y[k] (P1) or y[16 k], times the column weights
+// cw, as f32x2 of the high and of the low words.  nk: valid k; live: it is an
+// output.
 template <bool P1>
 __device__ __forceinline__ void zc_y_frag(const float2 *__restrict__ y, int k, int nk, bool live,
-                                          float sc, uint64_t (&h)[2], uint64_t (&l)[2]) {
+                                          const float *cw, uint64_t (&h)[2], uint64_t (&l)[2]) {
   float2 v[4];
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const int ku = k + (u & 1) + 8 * (u >> 1);
     v[u] = live && ku < nk ? y[ku * (P1 ? 1 : 16)] : make_float2(0.f, 0.f);
   }
-  const uint64_t s2 = f2_pk(sc, sc);
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
-    h[u] = f2_mul(f2_pk(v[2 * u].x, v[2 * u + 1].x), s2);
-    l[u] = f2_mul(f2_pk(v[2 * u].y, v[2 * u + 1].y), s2);
+    const float2 w = *reinterpret_cast<const float2 *>(cw + k + 8 * u);
+    const uint64_t w2 = f2_pk(w.x, w.y);
+    h[u] = f2_mul(f2_pk(v[2 * u].x, v[2 * u + 1].x), w2);
+    l[u] = f2_mul(f2_pk(v[2 * u].y, v[2 * u + 1].y), w2);
   }
 }
 
@@ -153,12 +158,12 @@ __device__ __forceinline__ void zc_exchange(uint32_t ta, uint64_t (&v)[N], bool 
   }
 }
 
-// Y-warp view of a job: its Y pairs, sizes, and each column block's G size,
-// piece and first 16-column block of Y.
+// Y loader's view of a job: its Y pairs, sizes, and each column block's G size
+// and first 16-column block of Y.
 struct ZcYJob {
   const float2 *Y2;
   int64_t czrow0;
-  int pA, na, nb, mtz, q, nblk, ng0, ng1, cb0, cb1, pc0, pc1;
+  int pA, nb, mtz, q, ng0, ng1, cb0, cb1;
 };
 
 __device__ __forceinline__ void zc_y_job(const SplitShared &S, const SplitWave &W, int jbeg,
@@ -167,15 +172,11 @@ __device__ __forceinline__ void zc_y_job(const SplitShared &S, const SplitWave &
   const WorkItem it = S.items[jb.w];
   Y.Y2 = reinterpret_cast<const float2 *>(W.scratch + W.y2_off[(int)(jb.w - W.w0)]);
   Y.pA = S.nabf[it.a];
-  Y.na = S.nao[it.a];
   Y.nb = S.nao[it.b];
-  Y.mtz = zc_tiles(Y.pA, Y.na);
-  Y.q = zc_rows_of(Y.na).q;
+  Y.mtz = zc_tiles(Y.pA, S.nao[it.a]);
+  Y.q = zc_rows_of(S.nao[it.a]).q;
   Y.czrow0 = S.czw_rowpre[it.a];
-  Y.nblk = jb.nblk;
   Y.ng0 = Y.ng1 = Y.cb0 = Y.cb1 = 0;
-  Y.pc0 = jb.piece[0];
-  Y.pc1 = jb.piece[1];
   if (jb.nblk > 0) {
     Y.ng0 = S.nao[S.nbr[it.gbase + jb.g[0]].other];
     Y.cb0 = S.kofs[it.gbase + jb.g[0]] / 16;
@@ -192,7 +193,7 @@ template <int KS, int NST, int YB>
 __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave W, ZcCfg cfg) {
   constexpr int NTM = 4;               // groups of 8 outputs
   constexpr int NV = NTM * 2 * 2;      // f32x2 accumulators of a thread
-  constexpr int YH = YB > 0 ? YB : 1;  // buffers of the Y warps' handshake
+  constexpr int YH = YB > 0 ? YB : 1;  // buffers of the Y loader's handshake
   constexpr int YPAD = ZC_YPAD;
   constexpr int A_BYTES = KS * 128 * 16 * 2;
   constexpr int B_BYTES = KS * ZC_COLS * 16 * 2;
@@ -219,7 +220,6 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
       umma::mbar_init(&ctl->tfull[b], 1);
       umma::mbar_init(&ctl->tempty[b], ZC_EPI);
       umma::mbar_init(&ctl->yfull[b], 1);
-      umma::mbar_init(&ctl->yrdy[b], 2);
       umma::mbar_init(&ctl->yempty[b], ZC_EPI);
     }
     umma::mbar_init(&ctl->drain, 1);
@@ -244,12 +244,9 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
     // ------------------------------------------------------------ A / B loader
     zc_loader<KS, NST, true, true>(S, W, cfg.jbeg, ncj, npair, smem, ctl->full, ctl->empty, abort_f,
                                    lane);
-  } else if (warp >= ZC_EPI + 2) {
-    // ------------------------------------------------------------ Y warps
-    // the first copies each tile's Y rows (and its row exponents) into a shared
-    // buffer; then both
-    // write the exponents of the al's Y, each for every other al
-    const int me = warp - (ZC_EPI + 2);
+  } else if (warp == ZC_EPI + 2) {
+    // ------------------------------------------------------------ Y loader
+    // each tile's Y rows and row exponents (with Y in global memory only these)
     long long hand = 0;
     bool ok = true;
     for (int p = 0; p < npair && ok; ++p) {
@@ -271,66 +268,46 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
         }
         const int tb = (int)(hand % YH);
         const long long use = hand / YH;
-        ++hand;
-        const int al0 = mt * Y.q, nal = min(Y.q, Y.pA - al0);
-        const int ncb0 = (Y.ng0 + 15) / 16, ncb1 = (Y.ng1 + 15) / 16;
-        const int ystr = Y.nb * 16 + YPAD;  // staged pairs per al
         bool w = true;
-        // the buffer (or, with Y in global memory, its exponents) is free
-        if (lane == 0 && (me == 0 || YB == 0)) {
+        if (lane == 0) {  // the buffer is free
           if (use >= 1)
             w = umma::mbar_wait(&ctl->yempty[tb], (uint32_t)((use - 1) & 1), S.err, ZC_WAIT);
           w = w && !*abort_f;
         }
-        w = __shfl_sync(0xffffffffu, (int)w, 0) != 0;
-        if constexpr (YB > 0) {
-          if (w && me == 0) {
-            umma::fence_proxy_async_smem();  // exponent bytes written here before
-            const uint32_t run = (uint32_t)(Y.nb * 16 * 8);  // one al's [b][16] pairs
-            const int n0 = ncb0 * nal, ncopy = n0 + ncb1 * nal;
-            if (lane == 0) {
-              umma::mbar_arrive_expect_tx(&ctl->yfull[tb], (uint32_t)ncopy * run + 256);
-              umma::bulk_g2s(ctl->erow[tb], S.cz_e + Y.czrow0 + mt * 128, 256, &ctl->yfull[tb]);
-            }
-            __syncwarp();
-            for (int q = lane; q < ncopy; q += 32) {
-              const int b = q < n0 ? 0 : 1;
-              const int r = q - (b ? n0 : 0), k = r / nal, al = al0 + r - k * nal;
-              umma::bulk_g2s(ybuf + tb * cfg.ybytes + (int64_t)q * ystr * 8,
-                             zc_y_global(Y.Y2, (b ? Y.cb1 : Y.cb0) + k, Y.pA, Y.nb, al), run,
-                             &ctl->yfull[tb]);
-            }
-          }
-          if (w && lane == 0)
-            w = umma::mbar_wait(&ctl->yfull[tb], (uint32_t)(use & 1), S.err, ZC_WAIT) && !*abort_f;
-          w = __shfl_sync(0xffffffffu, (int)w, 0) != 0;
-        }
-        if (!w) {
+        if (!__shfl_sync(0xffffffffu, (int)w, 0)) {
           if (lane == 0) *abort_f = 1;
           ok = false;
           break;
         }
-        for (int q = me; q < Y.nblk * nal; q += 2) {
-          const int b = q < nal ? 0 : 1, r = q - b * nal;
-          const int ng = b ? Y.ng1 : Y.ng0;
-          if constexpr (YB > 0) {
-            float2 *y = reinterpret_cast<float2 *>(ybuf + tb * cfg.ybytes) +
-                        (int64_t)((b ? ncb0 * nal : 0) + r) * ystr;
-            const int e = zc_y_exp(y, (int64_t)nal * ystr, Y.nb, ng, lane);
-            if (lane == 0) *reinterpret_cast<int *>(y + Y.nb * 16) = e;
-          } else {
-            const int e = zc_y_exp(zc_y_global(Y.Y2, b ? Y.cb1 : Y.cb0, Y.pA, Y.nb, al0 + r),
-                                   (int64_t)Y.pA * Y.nb * 16, Y.nb, ng, lane);
-            if (lane == 0) reinterpret_cast<int *>(ybuf)[b * 128 + r] = e;
+        ++hand;
+        if constexpr (YB > 0) {
+          const int al0 = mt * Y.q, nal = min(Y.q, Y.pA - al0);
+          const int ystr = Y.nb * 16 + YPAD;             // staged pairs per al
+          const uint32_t run = (uint32_t)(Y.nb * 16 * 8);  // one al's [b][16] pairs
+          const int n0 = (Y.ng0 + 15) / 16 * nal, ncopy = n0 + (Y.ng1 + 15) / 16 * nal;
+          if (lane == 0) {
+            umma::mbar_arrive_expect_tx(&ctl->yfull[tb], (uint32_t)ncopy * run + 256);
+            umma::bulk_g2s(ctl->erow[tb], S.cz_e + Y.czrow0 + mt * 128, 256, &ctl->yfull[tb]);
           }
-        }
-        if constexpr (YB > 0) umma::fence_proxy_async_smem();
-        else if (me == 0)
+          __syncwarp();
+          for (int q = lane; q < ncopy; q += 32) {
+            const int b = q < n0 ? 0 : 1;
+            const int r = q - (b ? n0 : 0), k = r / nal, al = al0 + r - k * nal;
+            umma::bulk_g2s(ybuf + tb * cfg.ybytes + (int64_t)q * ystr * 8,
+                           zc_y_global(Y.Y2, (b ? Y.cb1 : Y.cb0) + k, Y.pA, Y.nb, al), run,
+                           &ctl->yfull[tb]);
+          }
+        } else {
           for (int r = lane; r < 128; r += 32) ctl->erow[tb][r] = S.cz_e[Y.czrow0 + mt * 128 + r];
-        __syncwarp();
-        if (lane == 0) umma::mbar_arrive(&ctl->yrdy[tb]);
+          __syncwarp();
+          if (lane == 0) umma::mbar_arrive(&ctl->yfull[tb]);
+        }
       }
     }
+    // copies of tiles that nobody waits for any more after a failure elsewhere
+    if (YB > 0 && lane == 0)
+      for (long long t = max(0ll, hand - YH); t < hand; ++t)
+        umma::mbar_wait(&ctl->yfull[t % YH], (uint32_t)((t / YH) & 1), S.err, ZC_WAIT);
   } else if (warp == ZC_EPI + 1) {
     // ------------------------------------------------------------ MMA issuer
     if (lane == 0) {
@@ -426,26 +403,26 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
         if (warp == 0 || pr.two)
           zc_epi_job<true>(S, W, cfg.jbeg, warp ? pr.r1 : pr.r0, lane, ctl->ej[pp][warp]);
       } else if (warp < 8 && q4 >= 2 && (q4 == 2 || pr.two)) {
-        zc_epi_ecol<ZC_CW>(S, W, cfg.jbeg, q4 == 3 ? pr.r1 : pr.r0, hf, lane, ctl->ecol[q4 - 2]);
+        const int e = zc_col_exp<ZC_CW>(S, W, cfg.jbeg, q4 == 3 ? pr.r1 : pr.r0, hf, lane);
+        const int m = __reduce_max_sync(0xffffffffu, e);
+        if (lane < ZC_CW) ctl->cw[q4 - 2][hf * ZC_CW + lane] = zc_exp2(e - m);
+        if (lane == 0) ctl->emax[q4 - 2][hf] = m;
       }
       asm volatile("bar.sync 1, %0;" ::"r"(ZC_ET) : "memory");
       pr.m0 = ctl->ej[pp][0].mtz;
       if (pr.two) pr.m1 = ctl->ej[pp][1].mtz;
       // sums of the current tile's job over its tiles, one per (row, output) of
-      // this warp, in units of 2^E as f32 pairs: [output group][row half], high
-      // words then low words; the pair's other job keeps its own in spare TMEM
-      // columns
+      // this warp, as f32 pairs: [output group][row half], high words then low
+      // words; the pair's other job keeps its own in spare TMEM columns
       uint64_t acc[NV];
 #pragma unroll
       for (int k = 0; k < NV; ++k) acc[k] = 0;
-      int E = ZC_NOEXP, oE = ZC_NOEXP;
       bool parked = false, bad = false;
       int cur = 0, x, mt;
       while (pr.next(x, mt)) {
         if (x != cur) {
           zc_exchange<NV>(tpark, acc, parked);
           parked = true;
-          zc_swap(E, oE);
           cur = x;
         }
         const ZcEpiJob &ej = ctl->ej[pp][x];
@@ -501,8 +478,7 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
           __syncwarp();
           if (lane == 0) umma::mbar_arrive(&ctl->tempty[tb]);
         }
-        if constexpr (YB > 0) wait(&ctl->yfull[yt], ypar);
-        wait(&ctl->yrdy[yt], ypar);
+        wait(&ctl->yfull[yt], ypar);
         const int nal = min(ej.q, ej.pA - mt * ej.q);
         // the al [alf, ale) whose rows this fragment holds, and those of this
         // lane's two rows (-1: none)
@@ -513,8 +489,7 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
           const int hq = hb > 0 ? 1 : 0, nb = ej.nb;
           const int no = ej.nout[hq], cend = min(ZC_CW, ej.ncv[hq] - c0);
           const bool p1 = ej.pc[hq] == 1;
-          // Y of al in 16-column block k of this warp's block ([b][16] pairs),
-          // and its exponent
+          // Y of al in 16-column block k of this warp's block ([b][16] pairs)
           auto yrow = [&](int k, int al) -> const float2 * {
             if constexpr (YB > 0)
               return reinterpret_cast<const float2 *>(ybuf + yt * cfg.ybytes) +
@@ -523,55 +498,35 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
               return zc_y_global(reinterpret_cast<const float2 *>(W.scratch + ej.y2off),
                                  ej.gcb[hq] + k, ej.pA, nb, mt * ej.q + al);
           };
-          auto yexp = [&](int al) -> int {
-            if constexpr (YB > 0)
-              return *reinterpret_cast<const int *>(yrow(0, al) + nb * 16);
-            else
-              return reinterpret_cast<const int *>(ybuf)[hq * 128 + al];
-          };
-          // Z = (order-group sum) 2^(row + column exponent - SH) as f32 pairs;
-          // zero past the block's columns and in rows that hold no al
-          const int *ecol = ctl->ecol[x] + hf * ZC_CW;
-          int need = ZC_NOEXP, ey[2], alr[2], eA[2];
+          // Z = raw 2^(row exponent - SH + column exponent), raw as f32 pairs; raw is
+          // zero past the block's columns and in rows that hold no al, as the
+          // operands are.  Its digits, with an exponent per row (over this warp's
+          // columns), and each row's al (-1: none) and exponent in all
+          const float *cw = ctl->cw[x] + hf * ZC_CW;
+          int alr[2], er[2];
+          uint32_t zm[2] = {0, 0};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const uint64_t r = zl[j];
+            zl[j] = 0;
+            df_acc2(zh[j], zl[j], r);
+            zm[j & 1] = max(zm[j & 1], zc_max_abs(zh[j]));
+          }
+          float zs[2];
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             const int sl = ((rr + 8 * h + lr) * ej.inv) >> 16;
             alr[h] = sl < ej.slots && alb + sl < nal ? alb + sl : -1;
-            ey[h] = alr[h] >= 0 ? yexp(alr[h]) : -128;
-            eA[h] = ctl->erow[yt][r0 + 8 * h + lr] - SH;
+            zm[h] = max(zm[h], __shfl_xor_sync(0xffffffffu, zm[h], 1));
+            zm[h] = max(zm[h], __shfl_xor_sync(0xffffffffu, zm[h], 2));
+            er[h] = zc_exp_of(zm[h], zs[h]) + ctl->erow[yt][r0 + 8 * h + lr] - SH +
+                    ctl->emax[x][hf];
           }
-          float zm[2] = {0.f, 0.f};
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int h = j & 1, c = kc + 8 * (j >> 1);
-            float2 z0, z1;
-            df_fin2(zh[j], zl[j], eA[h] + ecol[c], eA[h] + ecol[c + 1], z0, z1);
-            if (ey[h] == -128 || c >= cend) z0 = make_float2(0.f, 0.f);
-            if (ey[h] == -128 || c + 1 >= cend) z1 = make_float2(0.f, 0.f);
-            zm[h] = fmaxf(zm[h], fmaxf(fabsf(z0.x), fabsf(z1.x)));
-            if (z0.x != z0.x || z1.x != z1.x) zm[h] = INFINITY;  // NaN stays
-            zh[j] = f2_pk(z0.x, z1.x);
-            zl[j] = f2_pk(z0.y, z1.y);
-          }
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-            if (zm[h] != 0.f) need = max(need, (int)(__float_as_uint(zm[h]) >> 23) - 126 + ey[h]);
-          need = __reduce_max_sync(0xffffffffu, need);
-          if (need > E) {  // a larger product: the sums move to its scale, with room to spare
-            const float sc = zc_exp2(E - need - 1);
-            const uint64_t s2 = f2_pk(sc, sc);
-#pragma unroll
-            for (int k = 0; k < NV; ++k) acc[k] = f2_mul(acc[k], s2);
-            E = need + 1;
-          }
-          if (need > ZC_NOEXP) {  // else nothing but zeros
-            // the rows' digits: Z 2^(ey - E), so that digit products of every al
-            // have the scale 2^E
+          if (__any_sync(0xffffffffu, (zm[0] | zm[1]) != 0)) {  // else nothing but zeros
             uint32_t A[4][ZC_DIG];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-              const float sc = zc_exp2(min(ey[j & 1] - E, 126));
-              const uint64_t s2 = f2_pk(sc, sc), l = f2_mul(zl[j], s2);
+              const uint64_t s2 = f2_pk(zs[j & 1], zs[j & 1]), l = f2_mul(zl[j], s2);
               uint64_t h = f2_mul(zh[j], s2);
 #pragma unroll
               for (int i = 0; i < ZC_DIG; ++i) A[j][i] = zc_digit(i, h, l);
@@ -585,24 +540,44 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
 #pragma unroll
                 for (int k = 0; k < 4; ++k) cg[g][k] = 0.f;
               const int o = nt * 8 + lr;
+              // exponents of Y for this lane's sums: rows h, outputs 2 (lane % 4) + {0, 1}
+              int ey[2][2] = {{0, 0}, {0, 0}};
               for (int al = alf; al < ale; ++al) {
-                const int e = yexp(al);
-                if (e == -128) continue;
                 uint64_t bh[2], bl[2];
-                const float sc = zc_exp2(-e);
                 if (p1)  // out b = o: Y[al][b][G, g = c0 + k]
-                  zc_y_frag<true>(yrow(c0 >> 4, al) + o * 16, kc, cend, o < no, sc, bh, bl);
+                  zc_y_frag<true>(yrow(c0 >> 4, al) + o * 16, kc, cend, o < no, cw, bh, bl);
                 else  // out g = o: Y[al][b = c0 + k][G, g]
-                  zc_y_frag<false>(yrow(nt >> 1, al) + c0 * 16 + (o & 15), kc, cend, o < no, sc,
+                  zc_y_frag<false>(yrow(nt >> 1, al) + c0 * 16 + (o & 15), kc, cend, o < no, cw,
                                    bh, bl);
-                const uint32_t k0 = alr[0] == al ? ~0u : 0u, k1 = alr[1] == al ? ~0u : 0u;
+                uint32_t m = max(zc_max_abs(bh[0]), zc_max_abs(bh[1]));
+                m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+                m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+                float ys;
+                const int e = zc_exp_of(m, ys);
+                const int e0 = __shfl_sync(0xffffffffu, e, 8 * (lane & 3));
+                const int e1 = __shfl_sync(0xffffffffu, e, 8 * (lane & 3) + 4);
+                const uint64_t s2 = f2_pk(ys, ys);
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                  bh[u] = f2_mul(bh[u], s2);
+                  bl[u] = f2_mul(bl[u], s2);
+                }
+                uint32_t kp[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                  kp[h] = alr[h] == al ? ~0u : 0u;
+                  if (alr[h] == al) {
+                    ey[h][0] = e0;
+                    ey[h][1] = e1;
+                  }
+                }
 #pragma unroll
                 for (int jd = 0; jd < ZC_DIG; ++jd) {
                   const uint32_t b0 = zc_digit(jd, bh[0], bl[0]), b1 = zc_digit(jd, bh[1], bl[1]);
 #pragma unroll
                   for (int i = 0; i < ZC_DIG - jd; ++i)
-                    zc_mma(cg[i + jd], A[0][i] & k0, A[1][i] & k1, A[2][i] & k0, A[3][i] & k1, b0,
-                           b1);
+                    zc_mma(cg[i + jd], A[0][i] & kp[0], A[1][i] & kp[1], A[2][i] & kp[0],
+                           A[3][i] & kp[1], b0, b1);
                 }
               }
               // order groups into the sums: the first three exactly (TwoSum), the
@@ -610,13 +585,14 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
 #pragma unroll
               for (int h = 0; h < 2; ++h) {
                 const int k = nt * 2 + h;
+                const uint64_t sc = f2_pk(zc_exp2(er[h] + ey[h][0]), zc_exp2(er[h] + ey[h][1]));
                 uint64_t t[ZC_DIG];
 #pragma unroll
                 for (int g = 0; g < ZC_DIG; ++g) t[g] = f2_pk(cg[g][2 * h], cg[g][2 * h + 1]);
-                uint64_t lo = f2_add(acc[NV / 2 + k], f2_add(t[3], f2_add(t[4], t[5])));
-                df_acc2(acc[k], lo, t[2]);
-                df_acc2(acc[k], lo, t[1]);
-                df_acc2(acc[k], lo, t[0]);
+                uint64_t lo =
+                    f2_fma(f2_add(t[3], f2_add(t[4], t[5])), sc, acc[NV / 2 + k]);
+#pragma unroll
+                for (int g = 2; g >= 0; --g) df_acc2(acc[k], lo, f2_mul(t[g], sc));
                 acc[NV / 2 + k] = lo;
               }
             }
@@ -645,9 +621,6 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
           qm[1] |= (bq == 1 ? 1u : 0u) << q;
         }
         bool inrange = true;
-        // 2^E in two steps: E may be below the normal range
-        const int e = max(E, -250), e1 = e / 2;
-        const float s1 = zc_exp2(e1), s2 = zc_exp2(e - e1);
 #pragma unroll
         for (int pass = 0; pass < NTM; ++pass) {
           if (pass >= npass) break;
@@ -656,8 +629,8 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
             const int k = pass * 2 + h;
             const float2 vh = f2_un(acc[k]), vl = f2_un(acc[NV / 2 + k]);
             float2 *o = red + (hf * ZC_PASS + kc) * 128 + r0 + 8 * h + lr;
-            o[0] = make_float2(vh.x * s1 * s2, vl.x * s1 * s2);
-            o[128] = make_float2(vh.y * s1 * s2, vl.y * s1 * s2);
+            o[0] = make_float2(vh.x, vl.x);
+            o[128] = make_float2(vh.y, vl.y);
           }
           asm volatile("bar.sync 1, %0;" ::"r"(ZC_ET) : "memory");
           for (int idx = et; idx < nown; idx += ZC_ET) {
@@ -688,7 +661,6 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
         if (!inrange) atomicOr(S.err, HFX_DEV_ERR_BOUNDS);
 #pragma unroll
         for (int k = 0; k < NV; ++k) acc[k] = 0;
-        E = ZC_NOEXP;
       }
     }
   }
@@ -726,7 +698,7 @@ cudaError_t zcw_run_t(const SplitShared &S, const SplitWave &W, int ybytes, int 
   cudaError_t e = launch(k_zcw<KS, 4, 2>, 4, 2, ybytes, true);
   if (e == cudaErrorMemoryAllocation) e = launch(k_zcw<KS, 5, 1>, 5, 1, ybytes, true);
   if (e == cudaErrorMemoryAllocation) e = launch(k_zcw<KS, 3, 1>, 3, 1, ybytes, true);
-  if (e == cudaErrorMemoryAllocation) e = launch(k_zcw<KS, 5, 0>, 5, 1, 2 * 128 * 4, false);
+  if (e == cudaErrorMemoryAllocation) e = launch(k_zcw<KS, 5, 0>, 5, 0, 0, false);
   return e;
 }
 

@@ -161,11 +161,10 @@ __device__ __forceinline__ void zc_epi_job(const SplitShared &S, const SplitWave
   }
 }
 
-// Column exponents of job r's column group hf (CW columns), by lanes < CW.
+// Exponent of column `lane` of job r's column group hf (CW columns; -1000: none).
 template <int CW>
-__device__ __forceinline__ void zc_epi_ecol(const SplitShared &S, const SplitWave &W, int jbeg,
-                                            int r, int hf, int lane, int *ecol) {
-  if (lane >= CW) return;
+__device__ __forceinline__ int zc_col_exp(const SplitShared &S, const SplitWave &W, int jbeg,
+                                          int r, int hf, int lane) {
   const ZcJob jb = zc_job(W, jbeg, r);
   const WorkItem it = S.items[jb.w];
   int ncv0 = 0, R0b = 16;
@@ -175,15 +174,11 @@ __device__ __forceinline__ void zc_epi_ecol(const SplitShared &S, const SplitWav
   }
   int c0 = 0;
   const int hb = zc_group_block<CW>(jb.nblk, R0b, hf, c0);
-  int e = -1000;
-  if (hb >= 0) {
-    const int pc = hb ? jb.piece[1] : jb.piece[0], g = hb ? jb.g[1] : jb.g[0];
-    const int at = pc == 1 ? S.nbr[it.gbase + g].other : it.b;
-    const int ncvh = S.nao[at];  // piece 1: nao(G); piece 2: nao(B)
-    const int cc = c0 + lane;
-    if (cc < ncvh) e = row_exponent((long long)S.de[S.aoff[at] + cc]);
-  }
-  ecol[hf * CW + lane] = e;
+  if (hb < 0 || lane >= CW) return -1000;
+  const int pc = hb ? jb.piece[1] : jb.piece[0], g = hb ? jb.g[1] : jb.g[0];
+  const int at = pc == 1 ? S.nbr[it.gbase + g].other : it.b;
+  // piece 1: nao(G) columns; piece 2: nao(B)
+  return c0 + lane < S.nao[at] ? row_exponent((long long)S.de[S.aoff[at] + c0 + lane]) : -1000;
 }
 
 // A launch's shared bytes of one staged Y buffer and its range of the job list.
