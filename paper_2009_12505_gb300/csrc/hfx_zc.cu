@@ -60,16 +60,13 @@ namespace split {
 
 constexpr int ZC_KMAX = 640;                     // K per job: exact f32 group sums
 
-// Epilogue geometry for EPI epilogue warps (8 or 16): 4 warps cover the 128
-// TMEM lanes, so there are EPI / 4 column groups of 32 / (EPI / 4) columns.
-template <int EPI>
-struct ZcGeo {
-  static constexpr int NQ = EPI / 4;                 // column groups
-  static constexpr int CW = ZC_COLS / NQ;            // Z columns per epilogue warp
-  static constexpr int ET = EPI * 32;                // epilogue threads
-  static constexpr int THREADS = (EPI + 3) * 32;     // + A/B loader, MMA issuer, Y loader
-  static constexpr int OWN = 2 * 32 * 32 / ET;       // owned outputs per epilogue thread
-};
+// Epilogue: 8 warps, one per TMEM lane quarter and column group of 16; a job's
+// block b is column group b.
+constexpr int ZC_EPI = 8;
+constexpr int ZC_NQ = 2;                      // column groups
+constexpr int ZC_CW = ZC_COLS / ZC_NQ;        // Z columns per epilogue warp
+constexpr int ZC_ET = ZC_EPI * 32;            // epilogue threads
+constexpr int ZC_THREADS = (ZC_EPI + 3) * 32;  // + A/B loader, MMA issuer, Y loader
 // Staged Y rows of one al are padded by ZC_YPAD pairs, so the rows of the
 // few al a warp touches fall in different shared-memory banks.
 constexpr int ZC_YPAD = 2;
@@ -532,11 +529,11 @@ __device__ __forceinline__ void zc_contract2(const uint64_t (&zh)[NP], const uin
   }
 }
 
-// Y-loader view of a job: its Y pairs, sizes and the 16-column blocks of Y
+// Y-loader view of a job: its Y pairs, sizes and the 16-column block of Y
 // columns of each column block.
 struct ZcYJob {
   const float2 *Y2;
-  int pA, na, nb, mtz, nblk, ncb0, ncb1, cb0, cb1;
+  int pA, na, nb, mtz, nblk, cb0, cb1;
 };
 
 __device__ __forceinline__ void zc_y_job(const SplitShared &S, const SplitWave &W, int jbeg,
@@ -547,24 +544,14 @@ __device__ __forceinline__ void zc_y_job(const SplitShared &S, const SplitWave &
   Y.pA = S.nabf[it.a];
   Y.na = S.nao[it.a];
   Y.nb = S.nao[it.b];
-  Y.mtz = (Y.pA * Y.na + 127) / 128;
+  Y.mtz = zc_row_tiles<false>(S, it.a);
   Y.nblk = jb.nblk;
-  Y.ncb0 = Y.ncb1 = Y.cb0 = Y.cb1 = 0;
-  if (jb.nblk > 0) {
-    Y.ncb0 = (S.nao[S.nbr[it.gbase + jb.g[0]].other] + 15) / 16;
-    Y.cb0 = S.kofs[it.gbase + jb.g[0]] / 16;
-  }
-  if (jb.nblk > 1) {
-    Y.ncb1 = (S.nao[S.nbr[it.gbase + jb.g[1]].other] + 15) / 16;
-    Y.cb1 = S.kofs[it.gbase + jb.g[1]] / 16;
-  }
+  Y.cb0 = jb.nblk > 0 ? S.kofs[it.gbase + jb.g[0]] / 16 : 0;
+  Y.cb1 = jb.nblk > 1 ? S.kofs[it.gbase + jb.g[1]] / 16 : 0;
 }
 
-template <int KS, int NST, int EPI, bool YST, bool PAIR>
-__global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
-    k_zc(SplitShared S, SplitWave W, ZcCfg cfg) {
-  constexpr int ZC_EPI = EPI, ZC_NQ = ZcGeo<EPI>::NQ, ZC_CW = ZcGeo<EPI>::CW,
-                ZC_ET = ZcGeo<EPI>::ET;
+template <int KS, int NST, bool YST, bool PAIR>
+__global__ void __launch_bounds__(ZC_THREADS, 1) k_zc(SplitShared S, SplitWave W, ZcCfg cfg) {
   // owned outputs per epilogue thread, for the job sums of both paired jobs: na x
   // (outputs of the job's blocks), at most 16 x 32
   constexpr int ZC_OWN = (16 * 32 + ZC_ET - 1) / ZC_ET;
@@ -657,15 +644,13 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
           const int al0 = mt * 128 / Y.na, al1 = min(Y.pA - 1, (mt * 128 + 127) / Y.na);
           const int nal = al1 - al0 + 1;
           const uint32_t run = (uint32_t)(Y.nb * 16 * 8);  // one al's [b][16] pairs
-          const int n0 = Y.ncb0 * nal, ncopy = n0 + (Y.nblk > 1 ? Y.ncb1 * nal : 0);
+          const int ncopy = Y.nblk * nal;
           if (lane == 0) umma::mbar_arrive_expect_tx(&ctl->yfull[tb], (uint32_t)ncopy * run);
           __syncwarp();
           for (int q = lane; q < ncopy; q += 32) {
-            const int b = q < n0 ? 0 : 1;
-            const int r = q - (b ? n0 : 0), k = r / nal, al = al0 + r - k * nal;
-            uint8_t *dst = ybuf + (tb * 2 + b) * cfg.ybytes +
-                           ((int64_t)(k * nal + (al - al0)) * (Y.nb * 16 + ZC_YPAD)) * 8;
-            umma::bulk_g2s(dst, zc_y_global(Y.Y2, (b ? Y.cb1 : Y.cb0) + k, Y.pA, Y.nb, al), run,
+            const int b = q < nal ? 0 : 1, r = q - b * nal;
+            uint8_t *dst = ybuf + (tb * 2 + b) * cfg.ybytes + (int64_t)r * (Y.nb * 16 + ZC_YPAD) * 8;
+            umma::bulk_g2s(dst, zc_y_global(Y.Y2, b ? Y.cb1 : Y.cb0, Y.pA, Y.nb, al0 + r), run,
                            &ctl->yfull[tb]);
           }
         }
@@ -677,75 +662,9 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
     }
   } else if (warp == ZC_EPI + 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      long long hand = 0;
-      int s = 0;  // operand slot and its parity
-      uint32_t ph = 0;
-      // N = R (KS - i) for a block of R rows (16 or 32), 16 KS at most 192
-      uint32_t idesc16[KS], idesc32[KS];
-#pragma unroll
-      for (int i = 0; i < KS; ++i) {
-        idesc16[i] = umma::idesc_bf16_f32(128, 16 * (KS - i));
-        idesc32[i] = umma::idesc_bf16_f32(128, 32 * (KS - i));
-      }
-      const uint32_t sbase = umma::smem_u32(smem);
-      bool ok = true;
-      for (int p = 0; p < npair && ok && !*abort_f; ++p) {
-        ZcPair<PAIR> pr;
-        pr.begin(p, ncj);
-        // entries, blocks and rows per block of the pair's two jobs
-        int ne0, nk0, R0, ne1 = 0, nk1 = 0, R1 = 16;
-        {
-          const ZcJob jb = zc_job(W, cfg.jbeg, pr.r0);
-          const WorkItem it = S.items[jb.w];
-          ne0 = jb.nent;
-          nk0 = jb.nblk;
-          R0 = zc_rows(S, jb, it);
-          pr.m0 = (S.nabf[it.a] * S.nao[it.a] + 127) / 128;
-        }
-        if (pr.two) {
-          const ZcJob jb = zc_job(W, cfg.jbeg, pr.r1);
-          const WorkItem it = S.items[jb.w];
-          ne1 = jb.nent;
-          nk1 = jb.nblk;
-          R1 = zc_rows(S, jb, it);
-          pr.m1 = (S.nabf[it.a] * S.nao[it.a] + 127) / 128;
-        }
-        int x, mt;
-        while (ok && !*abort_f && pr.next(x, mt)) {
-          const int nent = x ? ne1 : ne0, nblk = x ? nk1 : nk0, R = x ? R1 : R0;
-          const int tb = (int)(hand & 1);
-          const long long use = hand >> 1;
-          if (use >= 1 &&
-              !umma::mbar_wait(&ctl->tempty[tb], (uint32_t)((use - 1) & 1), S.err, ZC_WAIT)) {
-            ok = false;
-            break;
-          }
-          umma::fence_after_sync();
-          const uint32_t dcol = tbase + (uint32_t)(tb * 256);
-          for (int q = 0; q < nent; ++q) {
-            if (!umma::mbar_wait(&ctl->full[s], ph, S.err, ZC_WAIT)) {
-              ok = false;
-              break;
-            }
-            umma::fence_after_sync();
-            const uint32_t a0 = sbase + (uint32_t)(s * STG);
-            zc_stage_mmas<KS>(a0, a0 + A_BYTES, dcol, nblk, R, idesc16, idesc32, q == 0);
-            umma::mma_commit(&ctl->empty[s]);
-            if (++s == NST) {
-              s = 0;
-              ph ^= 1;
-            }
-          }
-          if (!ok) break;
-          umma::mma_commit(&ctl->tfull[tb]);
-          ++hand;
-        }
-      }
-      if (!ok) *abort_f = 1;
-      umma::mma_commit(&ctl->drain);
-      umma::mbar_wait(&ctl->drain, 0, S.err, ZC_WAIT);
-    }
+    if (lane == 0)
+      zc_issuer<KS, NST, false, PAIR>(S, W, cfg.jbeg, ncj, npair, smem, tbase, ctl->full,
+                                      ctl->empty, ctl->tfull, ctl->tempty, &ctl->drain, abort_f);
   } else {
     // ------------------------------------------------------------ epilogue
     const int q4 = warp & 3, hf = warp >> 2;  // TMEM lane quarter, column group
@@ -794,13 +713,10 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
         ++hand;
         // this row's exponent, read before the wait so its latency is hidden
         const int eA = (mt * 128 + row < pA * na) ? S.cz_e[ej.czrow0 + mt * 128 + row] : 0;
-        // this warp's column group: block hb, its first column c0
-        int c0 = 0;
-        const int hb = zc_group_block<ZC_CW>(ej.nblk, ej.R0b, hf, c0);
-        const int hq = hb > 0 ? 1 : 0;
+        // this warp's column group is block hf, if the job has it
+        const int hb = hf < ej.nblk ? hf : -1, hq = hb > 0 ? 1 : 0;
         const int piece = hb >= 0 ? ej.pc[hq] : 0;
-        const int Rh = hq ? 16 : ej.R0b;
-        const int noh = ej.nout[hq], ncvh = ej.ncv[hq], gcbh = ej.gcb[hq];
+        const int noh = ej.nout[hq], cend = ej.ncv[hq], gcbh = ej.gcb[hq];
         const int *ecol = ctl->ecol[x] + hf * ZC_CW;
         const float2 *Y2 = reinterpret_cast<const float2 *>(W.scratch + ej.y2off);
         bool okw = umma::mbar_wait(&ctl->tfull[tb], par, S.err, ZC_WAIT);
@@ -817,8 +733,7 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
         const int rowZ = mt * 128 + row;
         const bool rvalid = rowZ < pA * na;
         const int al = rvalid ? rowZ / na : 0;
-        const int al0 = mt * 128 / na, al1 = min(pA - 1, (mt * 128 + 127) / na);
-        const int nal = al1 - al0 + 1;
+        const int al0 = mt * 128 / na;
         // the order groups (exact f32 integers) summed in double-float, columns
         // (2j, 2j + 1) in the two f32x2 lanes
         constexpr int NP = ZC_CW / 2;
@@ -827,17 +742,15 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
         for (int j = 0; j < NP; ++j) ds[j] = dr[j] = 0;
         if (hb >= 0) {
           // the digit-order groups, three loads in flight per wait
-          // block hb's order g occupies TMEM columns hb 16 KS + g R .. + R
+          // block hb's order g occupies TMEM columns hb 16 KS + 16 g .. + 16
           const uint32_t ta = tbase + (uint32_t)(tb * 256) + ((uint32_t)(q4 * 32) << 16) +
-                              (uint32_t)(hb * 16 * KS + c0);
+                              (uint32_t)(hb * 16 * KS);
 #pragma unroll
           for (int g0 = 0; g0 < KS; g0 += 3) {
             uint32_t r[3][ZC_CW];
 #pragma unroll
             for (int u = 0; u < 3; ++u)
-              if (g0 + u < KS) {
-                umma::tmem_ld16_nowait(ta + (uint32_t)((g0 + u) * Rh), r[u]);
-              }
+              if (g0 + u < KS) umma::tmem_ld16_nowait(ta + (uint32_t)((g0 + u) * 16), r[u]);
             umma::tmem_wait_ld();
 #pragma unroll
             for (int u = 0; u < 3; ++u) {
@@ -855,13 +768,13 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
         umma::fence_before_sync();
         __syncwarp();
         if (lane == 0) umma::mbar_arrive(&ctl->tempty[tb]);
-        // Y rows of this thread's al in 16-column block k of G: [b][16] pairs
-        auto yrow = [&](int k) -> const float2 * {
+        // Y rows of this thread's al in block hb's columns: [b][16] pairs
+        auto yrow = [&]() -> const float2 * {
           if constexpr (YST)
             return reinterpret_cast<const float2 *>(ybuf + (tb * 2 + hb) * cfg.ybytes) +
-                   ((int64_t)k * nal + (al - al0)) * (nb * 16 + ZC_YPAD);
+                   (int64_t)(al - al0) * (nb * 16 + ZC_YPAD);
           else
-            return zc_y_global(Y2, gcbh + k, pA, nb, al);
+            return zc_y_global(Y2, gcbh, pA, nb, al);
         };
         // a tile of at most 32 valid rows (the last of an atom of 13 AOs and 60
         // ABFs holds 12): its rows are all in TMEM lane quarter 0, so that
@@ -876,7 +789,6 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
             for (int j = 0; j < NPT; ++j) {
               float2 z0, z1;
               df_fin2(ds[j], dr[j], eA + ecol[2 * j] - SH, eA + ecol[2 * j + 1] - SH, z0, z1);
-              const int cend = min(ZC_CW, ncvh - c0);
               zs[(2 * j) * 128] = 2 * j < cend ? z0 : make_float2(0.f, 0.f);
               zs[(2 * j + 1) * 128] = 2 * j + 1 < cend ? z1 : make_float2(0.f, 0.f);
             }
@@ -886,12 +798,7 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
           // takes the same operations as in the row-per-thread form below
           for (int idx = et; idx < ZC_NQ * 16 * 32; idx += ZC_ET) {
             const int r = idx & 31, qo = idx >> 5, q = qo >> 4, o = qo & 15;
-            int cq = 0;
-            const int bq = zc_group_block<ZC_CW>(ej.nblk, ej.R0b, q, cq);
-            if (r >= rv || bq < 0) continue;
-            const int bqi = bq > 0 ? 1 : 0;
-            if (o >= ej.nout[bqi]) continue;
-            const int cend = min(ZC_CW, ej.ncv[bqi] - cq);
+            if (r >= rv || q >= ej.nblk || o >= ej.nout[q]) continue;
             const float2 *zs = red + (int64_t)q * rs * 128 + 32 + r;
             uint64_t zh[NPT], nzh[NPT], nzl[NPT];
 #pragma unroll
@@ -902,18 +809,15 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
               nzl[j] = f2_pk(-z0.y, -z1.y);
             }
             const int alr = (mt * 128 + r) / na;
-            const float2 *yq = reinterpret_cast<const float2 *>(ybuf + (tb * 2 + bq) * cfg.ybytes);
+            const float2 *yb = reinterpret_cast<const float2 *>(ybuf + (tb * 2 + q) * cfg.ybytes) +
+                               (int64_t)(alr - al0) * (nb * 16 + ZC_YPAD);
             float2 *outp = red + ((int64_t)q * rs + o) * 128 + r;
-            if (ej.pc[bqi] == 1) {
-              const float2 *yb = yq + ((int64_t)(cq >> 4) * nal + (alr - al0)) * (nb * 16 + ZC_YPAD);
-              zc_contract2<NPT, true>(zh, nzh, nzl, cend, yb + (cq & 15) + o * 16, 1, outp);
-            } else {
-              const float2 *yb = yq + ((int64_t)(o >> 4) * nal + (alr - al0)) * (nb * 16 + ZC_YPAD);
-              zc_contract2<NPT, false>(zh, nzh, nzl, cend, yb + cq * 16 + (o & 15), 1, outp);
-            }
+            if (ej.pc[q] == 1)
+              zc_contract2<NPT, true>(zh, nzh, nzl, ej.ncv[q], yb + o * 16, 1, outp);
+            else
+              zc_contract2<NPT, false>(zh, nzh, nzl, ej.ncv[q], yb + o, 1, outp);
           }
         } else if (hb >= 0 && rvalid) {
-          const int cend = min(ZC_CW, ncvh - c0);
           float2 *rr = red + (int64_t)hf * rs * 128 + row;
           // Z = (order-group sum) 2^(eA + ecol - SH) as f32 pairs; zero from cend on
           float2 zp[NP][2];
@@ -933,26 +837,16 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
               nzh[j] = f2_pk(-zp[j][0].x, -zp[j][1].x);
               nzl[j] = f2_pk(-zp[j][0].y, -zp[j][1].y);
             }
-            if (piece == 1) {
-              // out b: Y[al][b][G, g = c0 + c]
-              zc_contract2<NP, true>(zh, nzh, nzl, cend, yrow(c0 >> 4) + (c0 & 15), noh, rr);
-            } else {
-              // out g: Y[al][b = c0 + c][G, g], one 16-column block of g at a time
-              for (int k = 0; 16 * k < noh; ++k)
-                zc_contract2<NP, false>(zh, nzh, nzl, cend, yrow(k) + c0 * 16,
-                                        min(16, noh - 16 * k), rr + 16 * k * 128);
-            }
+            if (piece == 1)  // out b: Y[al][b][G, g = c]
+              zc_contract2<NP, true>(zh, nzh, nzl, cend, yrow(), noh, rr);
+            else  // out g: Y[al][b = c][G, g]
+              zc_contract2<NP, false>(zh, nzh, nzl, cend, yrow(), noh, rr);
           } else {
             float2 z[ZC_CW];
 #pragma unroll
             for (int c = 0; c < ZC_CW; ++c) z[c] = zp[c >> 1][c & 1];
-            if (piece == 1) {
-              zc_contract<ZC_CW>(z, cend, yrow(c0 >> 4) + (c0 & 15), 16, 1, noh, rr);
-            } else {
-              for (int k = 0; 16 * k < noh; ++k)
-                zc_contract<ZC_CW>(z, cend, yrow(k) + c0 * 16, 1, 16, min(16, noh - 16 * k),
-                                   rr + 16 * k * 128);
-            }
+            if (piece == 1) zc_contract<ZC_CW>(z, cend, yrow(), 16, 1, noh, rr);
+            else zc_contract<ZC_CW>(z, cend, yrow(), 1, 16, noh, rr);
           }
         }
         __syncwarp();
@@ -960,18 +854,9 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
           if (lane == 0) umma::mbar_arrive(&ctl->yempty[tb]);
         }
         asm volatile("bar.sync 1, %0;" ::"r"(ZC_ET) : "memory");
-        // owners: (block, a, o) summed over the tile's rows (al, a) and the
-        // block's column groups, in a fixed order
+        // owners: (block, a, o) summed over the tile's rows (al, a) in a fixed order
         const int nout0 = ej.nout[0];
         const int own0 = na * nout0, nown = own0 + na * ej.nout[1];
-        unsigned qm0 = 0, qm1 = 0;  // column groups feeding block 0 and block 1 (bit q)
-#pragma unroll
-        for (int q = 0; q < ZC_NQ; ++q) {
-          int cq;
-          const int bq = zc_group_block<ZC_CW>(ej.nblk, ej.R0b, q, cq);
-          qm0 |= (bq == 0 ? 1u : 0u) << q;
-          qm1 |= (bq == 1 ? 1u : 0u) << q;
-        }
         const int r0 = mt * 128, rend = min(pA * na, r0 + 128);
         const int ph = r0 % na;
 #pragma unroll
@@ -981,23 +866,18 @@ __global__ void __launch_bounds__(ZcGeo<EPI>::THREADS, 1)
           const bool b1 = idx >= own0;
           const int rem = idx - (b1 ? own0 : 0);
           const int o = rem / na, a = rem - o * na;  // consecutive owners: consecutive a
-          const unsigned qm = b1 ? qm1 : qm0;
           int d = a - ph;
           if (d < 0) d += na;
           float h = jh[k], l = jl[k];
-#pragma unroll
-          for (int q = 0; q < ZC_NQ; ++q) {
-            if (!((qm >> q) & 1u)) continue;
-            const float2 *rq = red + ((int64_t)q * rs + o) * 128;
-            int lr = d;
-            // two rows per step: both loads in flight before the adds
-            for (; lr + na < rend - r0; lr += 2 * na) {
-              const float2 v0 = rq[lr], v1 = rq[lr + na];
-              df_add(h, l, v0);
-              df_add(h, l, v1);
-            }
-            if (lr < rend - r0) df_add(h, l, rq[lr]);
+          const float2 *rq = red + ((int64_t)(b1 ? 1 : 0) * rs + o) * 128;
+          int lr = d;
+          // two rows per step: both loads in flight before the adds
+          for (; lr + na < rend - r0; lr += 2 * na) {
+            const float2 v0 = rq[lr], v1 = rq[lr + na];
+            df_add(h, l, v0);
+            df_add(h, l, v1);
           }
+          if (lr < rend - r0) df_add(h, l, rq[lr]);
           jh[k] = h;
           jl[k] = l;
         }
@@ -1057,12 +937,12 @@ cudaError_t zc_range_t(const SplitShared &S, const SplitWave &W, int ybytes, int
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<blocks, ZcGeo<8>::THREADS, smem, st>>>(S, W, ZcCfg{yb, jbeg, jend, cta0});
+    kern<<<blocks, ZC_THREADS, smem, st>>>(S, W, ZcCfg{yb, jbeg, jend, cta0});
     return cudaGetLastError();
   };
-  if (smem_of(4, ybytes) <= kMax) return launch(k_zc<KS, 4, 8, true, true>, 4, ybytes);
-  if (smem_of(3, ybytes) <= kMax) return launch(k_zc<KS, 3, 8, true, false>, 3, ybytes);
-  return launch(k_zc<KS, 3, 8, false, false>, 3, 0);
+  if (smem_of(4, ybytes) <= kMax) return launch(k_zc<KS, 4, true, true>, 4, ybytes);
+  if (smem_of(3, ybytes) <= kMax) return launch(k_zc<KS, 3, true, false>, 3, ybytes);
+  return launch(k_zc<KS, 3, false, false>, 3, 0);
 }
 
 // Staged Y bytes of one block (al rows spanned by 128 (al, a) rows, all b, 2

@@ -310,75 +310,9 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
         umma::mbar_wait(&ctl->yfull[t % YH], (uint32_t)((t / YH) & 1), S.err, ZC_WAIT);
   } else if (warp == ZC_EPI + 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      long long hand = 0;
-      int s = 0;  // operand slot and its parity
-      uint32_t ph = 0;
-      // N = R (KS - i) for a block of R rows (16 or 32), 16 KS at most 192
-      uint32_t idesc16[KS], idesc32[KS];
-#pragma unroll
-      for (int i = 0; i < KS; ++i) {
-        idesc16[i] = umma::idesc_bf16_f32(128, 16 * (KS - i));
-        idesc32[i] = umma::idesc_bf16_f32(128, 32 * (KS - i));
-      }
-      const uint32_t sbase = umma::smem_u32(smem);
-      bool ok = true;
-      for (int p = 0; p < npair && ok && !*abort_f; ++p) {
-        ZcPair<true> pr;
-        pr.begin(p, ncj);
-        // entries, blocks and rows per block of the pair's two jobs
-        int ne0, nk0, R0, ne1 = 0, nk1 = 0, R1 = 16;
-        {
-          const ZcJob jb = zc_job(W, cfg.jbeg, pr.r0);
-          const WorkItem it = S.items[jb.w];
-          ne0 = jb.nent;
-          nk0 = jb.nblk;
-          R0 = zc_rows(S, jb, it);
-          pr.m0 = zc_tiles(S.nabf[it.a], S.nao[it.a]);
-        }
-        if (pr.two) {
-          const ZcJob jb = zc_job(W, cfg.jbeg, pr.r1);
-          const WorkItem it = S.items[jb.w];
-          ne1 = jb.nent;
-          nk1 = jb.nblk;
-          R1 = zc_rows(S, jb, it);
-          pr.m1 = zc_tiles(S.nabf[it.a], S.nao[it.a]);
-        }
-        int x, mt;
-        while (ok && !*abort_f && pr.next(x, mt)) {
-          const int nent = x ? ne1 : ne0, nblk = x ? nk1 : nk0, R = x ? R1 : R0;
-          const int tb = (int)(hand & 1);
-          const long long use = hand >> 1;
-          if (use >= 1 &&
-              !umma::mbar_wait(&ctl->tempty[tb], (uint32_t)((use - 1) & 1), S.err, ZC_WAIT)) {
-            ok = false;
-            break;
-          }
-          umma::fence_after_sync();
-          const uint32_t dcol = tbase + (uint32_t)(tb * 256);
-          for (int q = 0; q < nent; ++q) {
-            if (!umma::mbar_wait(&ctl->full[s], ph, S.err, ZC_WAIT)) {
-              ok = false;
-              break;
-            }
-            umma::fence_after_sync();
-            const uint32_t a0 = sbase + (uint32_t)(s * STG);
-            zc_stage_mmas<KS>(a0, a0 + A_BYTES, dcol, nblk, R, idesc16, idesc32, q == 0);
-            umma::mma_commit(&ctl->empty[s]);
-            if (++s == NST) {
-              s = 0;
-              ph ^= 1;
-            }
-          }
-          if (!ok) break;
-          umma::mma_commit(&ctl->tfull[tb]);
-          ++hand;
-        }
-      }
-      if (!ok) *abort_f = 1;
-      umma::mma_commit(&ctl->drain);
-      umma::mbar_wait(&ctl->drain, 0, S.err, ZC_WAIT);
-    }
+    if (lane == 0)
+      zc_issuer<KS, NST, true, true>(S, W, cfg.jbeg, ncj, npair, smem, tbase, ctl->full, ctl->empty,
+                                     ctl->tfull, ctl->tempty, &ctl->drain, abort_f);
   } else {
     // ------------------------------------------------------------ epilogue
     // TMEM lane quarter, column group, fragment of 16 rows

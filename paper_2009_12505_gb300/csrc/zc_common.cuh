@@ -81,11 +81,19 @@ __device__ __forceinline__ ZcJob zc_job(const SplitWave &W, int jbeg, int r) {
   return W.zc_jobs[jbeg + zc_job_of(r, blockIdx.x, gridDim.x)];
 }
 
-// rows of a job's lone column block (16 or 32); two blocks have 16 each
+// rows of a job's lone column block (16, in wide jobs also 32); two blocks have
+// 16 each
+template <bool WIDE>
 __device__ __forceinline__ int zc_rows(const SplitShared &S, const ZcJob &jb, const WorkItem &it) {
-  if (jb.nblk != 1) return 16;
+  if (!WIDE || jb.nblk != 1) return 16;
   const int ncb = jb.piece[0] == 1 ? S.nao[S.nbr[it.gbase + jb.g[0]].other] : S.nao[it.b];
   return ncb <= 16 ? 16 : 32;
+}
+
+// row tiles of atom a's A operand
+template <bool WIDE>
+__device__ __forceinline__ int zc_row_tiles(const SplitShared &S, int a) {
+  return WIDE ? zc_tiles(S.nabf[a], S.nao[a]) : (S.nabf[a] * S.nao[a] + 127) / 128;
 }
 
 // block and first column cq of column group q of width CW: two 16-column
@@ -141,7 +149,7 @@ __device__ __forceinline__ void zc_epi_job(const SplitShared &S, const SplitWave
     e.slots = R.slots;
     e.q = R.q;
     e.inv = (65536 + na - 1) / na;
-    e.mtz = WIDE ? zc_tiles(pA, na) : (pA * na + 127) / 128;
+    e.mtz = zc_row_tiles<WIDE>(S, it.a);
     e.czrow0 = (WIDE ? S.czw_rowpre : S.cz_rowpre)[it.a];
     e.nblk = jb.nblk;
     e.R0b = 16;
@@ -235,9 +243,8 @@ __device__ __forceinline__ void zc_ld_job(const SplitShared &S, const SplitWave 
   L.ent = jb.ent;
   L.nent = jb.nent;
   L.nblk = jb.nblk;
-  L.Rl = zc_rows(S, jb, it);
-  L.mtz = WIDE ? zc_tiles(S.nabf[it.a], S.nao[it.a])
-               : (S.nabf[it.a] * S.nao[it.a] + 127) / 128;
+  L.Rl = zc_rows<WIDE>(S, jb, it);
+  L.mtz = zc_row_tiles<WIDE>(S, it.a);
   L.held = -1;
   L.mine = ZcEnt{0, {-1, -1}};
 }
@@ -308,6 +315,80 @@ __device__ __forceinline__ void zc_loader(const SplitShared &S, const SplitWave 
   if (lane == 0)
     for (int t = ring.pending(); t < ring.step; ++t)
       umma::mbar_wait(&full[t % NST], (uint32_t)((t / NST) & 1), S.err, ZC_WAIT);
+}
+
+// The MMA issuer of both kernels, by one thread: every stage of the jobs' tiles
+// into the TMEM accumulators (two, 256 columns each) in turn.
+template <int KS, int NST, bool WIDE, bool PAIR>
+__device__ __forceinline__ void zc_issuer(const SplitShared &S, const SplitWave &W, int jbeg,
+                                          int ncj, int npair, uint8_t *smem, uint32_t tbase,
+                                          uint64_t *full, uint64_t *empty, uint64_t *tfull,
+                                          uint64_t *tempty, uint64_t *drain,
+                                          volatile int *abort_f) {
+  constexpr int A_BYTES = KS * 128 * 16 * 2;
+  constexpr int STG = A_BYTES + KS * ZC_COLS * 16 * 2;
+  long long hand = 0;
+  int s = 0;  // operand slot and its parity
+  uint32_t ph = 0;
+  // N = R (KS - i) for a block of R rows (16, in wide jobs also 32), at most 192
+  uint32_t idesc16[KS], idesc32[KS];
+#pragma unroll
+  for (int i = 0; i < KS; ++i) {
+    idesc16[i] = umma::idesc_bf16_f32(128, 16 * (KS - i));
+    idesc32[i] = umma::idesc_bf16_f32(128, 32 * (KS - i));
+  }
+  const uint32_t sbase = umma::smem_u32(smem);
+  bool ok = true;
+  for (int p = 0; p < npair && ok && !*abort_f; ++p) {
+    ZcPair<PAIR> pr;
+    pr.begin(p, ncj);
+    // entries, blocks and rows per block of the pair's two jobs
+    int ne[2] = {0, 0}, nk[2] = {0, 0}, R[2] = {16, 16}, mtz[2] = {0, 0};
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      if (j == 1 && !pr.two) break;
+      const ZcJob jb = zc_job(W, jbeg, j ? pr.r1 : pr.r0);
+      const WorkItem it = S.items[jb.w];
+      ne[j] = jb.nent;
+      nk[j] = jb.nblk;
+      R[j] = zc_rows<WIDE>(S, jb, it);
+      mtz[j] = zc_row_tiles<WIDE>(S, it.a);
+    }
+    pr.m0 = mtz[0];
+    pr.m1 = mtz[1];
+    int x, mt;
+    while (ok && !*abort_f && pr.next(x, mt)) {
+      const int nent = x ? ne[1] : ne[0], nblk = x ? nk[1] : nk[0], Rx = x ? R[1] : R[0];
+      const int tb = (int)(hand & 1);
+      const long long use = hand >> 1;
+      if (use >= 1 && !umma::mbar_wait(&tempty[tb], (uint32_t)((use - 1) & 1), S.err, ZC_WAIT)) {
+        ok = false;
+        break;
+      }
+      umma::fence_after_sync();
+      const uint32_t dcol = tbase + (uint32_t)(tb * 256);
+      for (int q = 0; q < nent; ++q) {
+        if (!umma::mbar_wait(&full[s], ph, S.err, ZC_WAIT)) {
+          ok = false;
+          break;
+        }
+        umma::fence_after_sync();
+        const uint32_t a0 = sbase + (uint32_t)(s * STG);
+        zc_stage_mmas<KS>(a0, a0 + A_BYTES, dcol, nblk, Rx, idesc16, idesc32, q == 0);
+        umma::mma_commit(&empty[s]);
+        if (++s == NST) {
+          s = 0;
+          ph ^= 1;
+        }
+      }
+      if (!ok) break;
+      umma::mma_commit(&tfull[tb]);
+      ++hand;
+    }
+  }
+  if (!ok) *abort_f = 1;
+  umma::mma_commit(drain);
+  umma::mbar_wait(drain, 0, S.err, ZC_WAIT);
 }
 
 }  // namespace split
