@@ -30,22 +30,21 @@
 // exponents.  Every wait is bounded; on expiry the kernel records HFX_DEV_ERR_TIMEOUT, drains its copies and MMAs,
 // frees TMEM and returns.
 //
-// What bounds it: the epilogue, beside up to 22 operand stages a tile; it also
-// waits for the single Y buffer (five operand stages leave no room for a second
-// one; three stages and two buffers took 116 ms where this took 109.7).  8-atom
+// What bounds it: the epilogue, beside up to 22 operand stages a tile.  8-atom
 // two-element cell (13/60 and 27/90, C, D to 9 bohr): 178.7 ms for its wide jobs
 // with a double-float contraction from global memory, 127 ms with that contraction
 // halved and Y staged, 109.7 ms with this product and two warps that looked for
-// one exponent per al before a tile could be read; with the exponents taken from
-// each fragment's own loads the whole step went from 144.5 to 134.5 ms (35 ms of
-// bf16 products at the sustained peak in this kernel).
+// one exponent per al before a tile could be read, 97.8 ms with the exponents taken
+// from each fragment's own loads (35 ms of bf16 products at the sustained peak).
 #include "zc_common.cuh"
 
 namespace split {
 
 // Epilogue: 16 warps, one per TMEM lane quarter, group of 16 columns and 16-row
 // fragment, so that each scheduler has four of them to hide latencies; with the
-// other roles a scheduler has five warps, which leaves 96 registers a thread.
+// other roles a scheduler has five warps, which leaves 96 registers a thread, too
+// few for the digits, order groups and sums at once: ptxas spills 572 bytes a
+// thread (952 of loads).
 constexpr int ZC_EPI = 16;
 constexpr int ZC_NQ = 2;                         // column groups
 constexpr int ZC_CW = ZC_COLS / ZC_NQ;           // Z columns per epilogue warp
@@ -58,11 +57,11 @@ constexpr int ZC_PASS = 8;   // outputs of a block per pass through the reductio
 constexpr int ZC_DIG = 6;    // digits of the second product's operands (8 bits each)
 
 struct ZcwSmem {
-  uint64_t full[8], empty[8], tfull[2], tempty[2], yfull[2], yempty[2], drain;
+  uint64_t full[8], empty[8], tfull[2], tempty[2], yfull, yempty, drain;
   unsigned long long t_start;  // globaltimer at the start of the roles
   uint32_t tslot;
   int abort_f;
-  __align__(16) int16_t erow[2][128];  // row exponents of the tile in each Y buffer
+  __align__(16) int16_t erow[128];  // row exponents of the tile that Y is staged for
   // column exponents of the pair's jobs: the largest of each column group, and
   // each column's 2^(exponent - largest) (column group q at q * CW)
   int emax[2][ZC_NQ];
@@ -187,21 +186,20 @@ __device__ __forceinline__ void zc_y_job(const SplitShared &S, const SplitWave &
   }
 }
 
-// NST operand stages; YB staged Y buffers (0: the epilogue reads Y from global
+// NST operand stages; YST: Y is staged (else the epilogue reads it from global
 // memory).
-template <int KS, int NST, int YB>
+template <int KS, int NST, bool YST>
 __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave W, ZcCfg cfg) {
   constexpr int NTM = 4;               // groups of 8 outputs
   constexpr int NV = NTM * 2 * 2;      // f32x2 accumulators of a thread
-  constexpr int YH = YB > 0 ? YB : 1;  // buffers of the Y loader's handshake
   constexpr int YPAD = ZC_YPAD;
   constexpr int A_BYTES = KS * 128 * 16 * 2;
   constexpr int B_BYTES = KS * ZC_COLS * 16 * 2;
   constexpr int STG = A_BYTES + B_BYTES;
   constexpr int SH = 7 * (KS + 1);
   extern __shared__ __align__(1024) uint8_t smem[];
-  uint8_t *ybuf = smem + NST * STG;                                    // [YH][ybytes]
-  float2 *red = reinterpret_cast<float2 *>(ybuf + YH * cfg.ybytes);    // [ZC_NQ][ZC_PASS][128]
+  uint8_t *ybuf = smem + NST * STG;                                  // [ybytes]
+  float2 *red = reinterpret_cast<float2 *>(ybuf + cfg.ybytes);       // [ZC_NQ][ZC_PASS][128]
   ZcwSmem *ctl = reinterpret_cast<ZcwSmem *>(red + ZC_NQ * ZC_PASS * 128);
   volatile int *abort_f = &ctl->abort_f;
 
@@ -219,9 +217,9 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
     for (int b = 0; b < 2; ++b) {
       umma::mbar_init(&ctl->tfull[b], 1);
       umma::mbar_init(&ctl->tempty[b], ZC_EPI);
-      umma::mbar_init(&ctl->yfull[b], 1);
-      umma::mbar_init(&ctl->yempty[b], ZC_EPI);
     }
+    umma::mbar_init(&ctl->yfull, 1);
+    umma::mbar_init(&ctl->yempty, ZC_EPI);
     umma::mbar_init(&ctl->drain, 1);
     ctl->abort_f = 0;
     umma::fence_barrier_init();
@@ -266,12 +264,10 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
           zc_swap(Y, Yo);
           cur = x;
         }
-        const int tb = (int)(hand % YH);
-        const long long use = hand / YH;
         bool w = true;
         if (lane == 0) {  // the buffer is free
-          if (use >= 1)
-            w = umma::mbar_wait(&ctl->yempty[tb], (uint32_t)((use - 1) & 1), S.err, ZC_WAIT);
+          if (hand >= 1)
+            w = umma::mbar_wait(&ctl->yempty, (uint32_t)((hand - 1) & 1), S.err, ZC_WAIT);
           w = w && !*abort_f;
         }
         if (!__shfl_sync(0xffffffffu, (int)w, 0)) {
@@ -280,34 +276,33 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
           break;
         }
         ++hand;
-        if constexpr (YB > 0) {
+        if constexpr (YST) {
           const int al0 = mt * Y.q, nal = min(Y.q, Y.pA - al0);
           const int ystr = Y.nb * 16 + YPAD;             // staged pairs per al
           const uint32_t run = (uint32_t)(Y.nb * 16 * 8);  // one al's [b][16] pairs
           const int n0 = (Y.ng0 + 15) / 16 * nal, ncopy = n0 + (Y.ng1 + 15) / 16 * nal;
           if (lane == 0) {
-            umma::mbar_arrive_expect_tx(&ctl->yfull[tb], (uint32_t)ncopy * run + 256);
-            umma::bulk_g2s(ctl->erow[tb], S.cz_e + Y.czrow0 + mt * 128, 256, &ctl->yfull[tb]);
+            umma::mbar_arrive_expect_tx(&ctl->yfull, (uint32_t)ncopy * run + 256);
+            umma::bulk_g2s(ctl->erow, S.cz_e + Y.czrow0 + mt * 128, 256, &ctl->yfull);
           }
           __syncwarp();
           for (int q = lane; q < ncopy; q += 32) {
             const int b = q < n0 ? 0 : 1;
             const int r = q - (b ? n0 : 0), k = r / nal, al = al0 + r - k * nal;
-            umma::bulk_g2s(ybuf + tb * cfg.ybytes + (int64_t)q * ystr * 8,
+            umma::bulk_g2s(ybuf + (int64_t)q * ystr * 8,
                            zc_y_global(Y.Y2, (b ? Y.cb1 : Y.cb0) + k, Y.pA, Y.nb, al), run,
-                           &ctl->yfull[tb]);
+                           &ctl->yfull);
           }
         } else {
-          for (int r = lane; r < 128; r += 32) ctl->erow[tb][r] = S.cz_e[Y.czrow0 + mt * 128 + r];
+          for (int r = lane; r < 128; r += 32) ctl->erow[r] = S.cz_e[Y.czrow0 + mt * 128 + r];
           __syncwarp();
-          if (lane == 0) umma::mbar_arrive(&ctl->yfull[tb]);
+          if (lane == 0) umma::mbar_arrive(&ctl->yfull);
         }
       }
     }
-    // copies of tiles that nobody waits for any more after a failure elsewhere
-    if (YB > 0 && lane == 0)
-      for (long long t = max(0ll, hand - YH); t < hand; ++t)
-        umma::mbar_wait(&ctl->yfull[t % YH], (uint32_t)((t / YH) & 1), S.err, ZC_WAIT);
+    // copies of a tile that nobody waits for any more after a failure elsewhere
+    if (YST && lane == 0 && hand > 0)
+      umma::mbar_wait(&ctl->yfull, (uint32_t)((hand - 1) & 1), S.err, ZC_WAIT);
   } else if (warp == ZC_EPI + 1) {
     // ------------------------------------------------------------ MMA issuer
     if (lane == 0)
@@ -361,8 +356,7 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
         }
         const ZcEpiJob &ej = ctl->ej[pp][x];
         const int tb = (int)(hand & 1);
-        const int yt = (int)(hand % YH);
-        const uint32_t ypar = (uint32_t)((hand / YH) & 1);
+        const uint32_t ypar = (uint32_t)(hand & 1);
         // this warp's column group: block hb, its first column c0
         int c0 = 0;
         const int hb = zc_group_block<ZC_CW>(ej.nblk, ej.R0b, hf, c0);
@@ -412,7 +406,7 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
           __syncwarp();
           if (lane == 0) umma::mbar_arrive(&ctl->tempty[tb]);
         }
-        wait(&ctl->yfull[yt], ypar);
+        wait(&ctl->yfull, ypar);
         const int nal = min(ej.q, ej.pA - mt * ej.q);
         // the al [alf, ale) whose rows this fragment holds, and those of this
         // lane's two rows (-1: none)
@@ -425,8 +419,8 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
           const bool p1 = ej.pc[hq] == 1;
           // Y of al in 16-column block k of this warp's block ([b][16] pairs)
           auto yrow = [&](int k, int al) -> const float2 * {
-            if constexpr (YB > 0)
-              return reinterpret_cast<const float2 *>(ybuf + yt * cfg.ybytes) +
+            if constexpr (YST)
+              return reinterpret_cast<const float2 *>(ybuf) +
                      (((hq ? ej.ncb0 : 0) + k) * nal + al) * (nb * 16 + YPAD);
             else
               return zc_y_global(reinterpret_cast<const float2 *>(W.scratch + ej.y2off),
@@ -453,7 +447,7 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
             alr[h] = sl < ej.slots && alb + sl < nal ? alb + sl : -1;
             zm[h] = max(zm[h], __shfl_xor_sync(0xffffffffu, zm[h], 1));
             zm[h] = max(zm[h], __shfl_xor_sync(0xffffffffu, zm[h], 2));
-            er[h] = zc_exp_of(zm[h], zs[h]) + ctl->erow[yt][r0 + 8 * h + lr] - SH +
+            er[h] = zc_exp_of(zm[h], zs[h]) + ctl->erow[r0 + 8 * h + lr] - SH +
                     ctl->emax[x][hf];
           }
           if (__any_sync(0xffffffffu, (zm[0] | zm[1]) != 0)) {  // else nothing but zeros
@@ -533,7 +527,7 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
           }
         }
         __syncwarp();
-        if (!bad && lane == 0) umma::mbar_arrive(&ctl->yempty[yt]);
+        if (!bad && lane == 0) umma::mbar_arrive(&ctl->yempty);
         if (mt + 1 < ej.mtz) continue;
         // the job's last tile: sum its rows (slots and column groups) in a fixed
         // order and add the finished blocks to Sigma (and mirrors); a sum
@@ -609,18 +603,20 @@ __global__ void __launch_bounds__(ZC_THREADS, 1) k_zcw(SplitShared S, SplitWave 
 }
 
 // Variants by what fits 227 KB next to the reduction buffer (16 KB) and the
-// operand stages (30 KB each with 6 digits).  The operand stream bounds the
-// kernel, so five stages with one Y buffer come before three with two (ab8
-// cell, 13 / 27 AOs); a system of 27-AO atoms alone has room for four and two.
-// Y is read from global memory beside atoms of very few AOs, whose row tiles
-// hold many al.
+// operand stages (30 KB each with 6 digits).  One Y buffer: a second one was slower
+// even where it fits beside four stages (6 digits, 27/90 alone: 10.1 against
+// 9.4 ms; 20/70 alone: 15.7 against 14.0).  Four stages and five take about the
+// same time (two-element cell, 13/60 and 27/90: 97.8 and 100.3 ms with 6 digits,
+// 82.1 and 83.5 with 4), so does the fallback of three (99.0, 84.6).  Y is read
+// from global memory (115.7 ms there) only beside atoms of very few AOs, whose row
+// tiles hold many al.
 template <int KS>
 cudaError_t zcw_run_t(const SplitShared &S, const SplitWave &W, int ybytes, int nsm, int jbeg,
                       int jend, int cta0, cudaStream_t st) {
   const int blocks = (int)std::min<int64_t>(jend - jbeg, nsm);
   if (blocks <= 0) return cudaSuccess;
-  auto launch = [&](auto kern, int nst, int nyb, int yb, bool probe) -> cudaError_t {
-    const size_t smem = (size_t)nst * KS * (128 + ZC_COLS) * 16 * 2 + (size_t)nyb * yb +
+  auto launch = [&](auto kern, int nst, int yb, bool probe) -> cudaError_t {
+    const size_t smem = (size_t)nst * KS * (128 + ZC_COLS) * 16 * 2 + (size_t)yb +
                         (size_t)ZC_NQ * ZC_PASS * 128 * sizeof(float2) + sizeof(ZcwSmem) + 64;
     if (probe && smem > 227 * 1024) return cudaErrorMemoryAllocation;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -629,10 +625,9 @@ cudaError_t zcw_run_t(const SplitShared &S, const SplitWave &W, int ybytes, int 
     kern<<<blocks, ZC_THREADS, smem, st>>>(S, W, ZcCfg{yb, jbeg, jend, cta0});
     return cudaGetLastError();
   };
-  cudaError_t e = launch(k_zcw<KS, 4, 2>, 4, 2, ybytes, true);
-  if (e == cudaErrorMemoryAllocation) e = launch(k_zcw<KS, 5, 1>, 5, 1, ybytes, true);
-  if (e == cudaErrorMemoryAllocation) e = launch(k_zcw<KS, 3, 1>, 3, 1, ybytes, true);
-  if (e == cudaErrorMemoryAllocation) e = launch(k_zcw<KS, 5, 0>, 5, 0, 0, false);
+  cudaError_t e = launch(k_zcw<KS, 4, true>, 4, ybytes, true);
+  if (e == cudaErrorMemoryAllocation) e = launch(k_zcw<KS, 3, true>, 3, ybytes, true);
+  if (e == cudaErrorMemoryAllocation) e = launch(k_zcw<KS, 5, false>, 5, 0, false);
   return e;
 }
 
