@@ -113,26 +113,45 @@ def workload_desc(wl) -> str:
 
 
 # dram__bytes_read.sum + dram__bytes_write.sum of one k_zc launch on the 8-atom
-# cell over its issued bf16 tensor flops, captured from the hfx_zc.cu whose code
-# (comments and blank space removed) has this sha256 prefix (see the k_zc
+# cell over its issued bf16 tensor flops (the build's own count), captured from
+# the hfx_zc.cu whose code, headers included, has this digest (see the k_zc
 # profile summary under profiles/)
-ZC_BYTES_PER_TENSOR_FLOP = (22.585361e9 + 0.377352e9) / 13.4e12
-ZC_CAPTURED_SHA = "b9c11dbd0960f869"
+ZC_BYTES_PER_TENSOR_FLOP = (22.434085888e9 + 0.377987840e9) / 13.417386737664e12
+ZC_CAPTURED_SHA = "bac28084c3f5d364"
 
 
 def source_digest(path):
-    """sha256 prefix of a C++/CUDA source's code: comments and blank space
+    """sha256 prefix of a C++/CUDA source's code and of the headers it includes
+    by quoted name, in order of their first use: comments and blank space
     removed, so an edit of comments alone keeps the digest."""
     import hashlib
     import re
-    text = open(path, encoding="utf-8").read()
-    text = re.sub(r"/\*.*?\*/", " ", text, flags=re.S)
-    text = re.sub(r"//[^\n]*", " ", text)
-    text = " ".join(text.split())
-    return hashlib.sha256(text.encode()).hexdigest()[:16]
+    seen, out = set(), []
+
+    def take(p):
+        p = os.path.realpath(p)
+        if p in seen:
+            return
+        seen.add(p)
+        text = open(p, encoding="utf-8").read()
+        text = re.sub(r"/\*.*?\*/", " ", text, flags=re.S)
+        text = re.sub(r"//[^\n]*", " ", text)
+        for inc in re.findall(r'^\s*#\s*include\s+"([^"]+)"', text, flags=re.M):
+            q = os.path.join(os.path.dirname(p), inc)
+            if os.path.exists(q):
+                take(q)
+        out.append(" ".join(text.split()))
+
+    take(path)
+    return hashlib.sha256("\n".join(out).encode()).hexdigest()[:16]
 
 
-def zc_traffic(tensor_flops_per_launch):
+def zc_traffic(tensor_flops_per_launch, max_nao=0):
+    """DRAM bytes of one k_zc launch, from its issued flops; None when the code
+    differs from the captured one, and for cells with atoms of more than 16 AOs,
+    whose products are k_zcw's too (never captured for this)."""
+    if max_nao > 16:
+        return None
     src = os.path.join(ROOT, "paper_2009_12505_gb300", "csrc", "hfx_zc.cu")
     try:
         sha = source_digest(src)
@@ -648,8 +667,11 @@ def run_gpu(args):
     # with the mirror pieces the D_FG / D_FB kernel also yields the D_AG piece
     canon = {"v1_DFG": cp[0] + cp[1] + (cp[2] if st["mirror"] else 0.0),
              "Y": st["canonical_flops_y"], "v4_DAB": cp[3]}
+    max_nao = int(wl.system.nao.max())
     desc = {"v1_DFG": "k_zc: D_FG + D_FB pieces (tcgen05 digit products, double-float Y "
-                      "contraction in the epilogue)",
+                      "contraction in the epilogue)" +
+                      ("; k_zcw for blocks of more than 16 AOs (Y contraction as a second digit "
+                       "product)" if max_nao > 16 else ""),
             "Y": "k_pgemm job 0: Y = V C (tcgen05 digit products)",
             "v4_DAB": "k_pgemm job 1: D_AB piece (tcgen05 digit products)"}
     if ktf.get(top, 0.0) == 0 or top not in canon:
@@ -677,11 +699,13 @@ def run_gpu(args):
                 "effective_tflops": canon[top] * args.steps / t_s / 1e12,
                 "effective_is": "canonical Algorithm 3 flops of the pieces the kernel yields "
                                 "/ its device time (counts work the reassociations avoid)",
-                "traffic": zc_traffic(ktf[top] / args.steps / nwaves) if top == "v1_DFG" else None,
+                "traffic": (zc_traffic(ktf[top] / args.steps / nwaves, max_nao)
+                            if top == "v1_DFG" else None),
                 "traffic_note": ("DRAM bytes per launch (one launch per wave): bytes per issued "
                                  "tensor flop from one ncu capture of this kernel on the 8-atom "
-                                 "cell, times this launch's issued flops; null once the kernel "
-                                 "source differs from the captured one") if top == "v1_DFG" else None}
+                                 "cell, times this launch's issued flops; null once the kernel's "
+                                 "code differs from the captured one, and for cells whose wide "
+                                 "blocks go to another kernel") if top == "v1_DFG" else None}
     roof["kernel_ms_per_step"] = {k: v / args.steps for k, v in kms.items()}
     roof["kernel_tensor_tflop_per_step"] = {k: v / args.steps / 1e12 for k, v in ktf.items() if v}
     roof["launches_per_step_of_top"] = nwaves

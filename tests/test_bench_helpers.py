@@ -26,6 +26,27 @@ def test_source_digest_ignores_comments_only(tmp_path):
     assert bench.source_digest(str(a)) != bench.source_digest(str(c))
 
 
+def test_source_digest_covers_the_headers(tmp_path):
+    (tmp_path / "sub").mkdir()
+    top, h, deep = tmp_path / "a.cu", tmp_path / "sub" / "h.cuh", tmp_path / "deep.h"
+    top.write_text('#include <vector>\n#include "sub/h.cuh"\n// #include "none.h"\nint a;\n')
+    h.write_text('#pragma once\n#include "../deep.h"\nint b;\n')
+    deep.write_text('#include "sub/h.cuh"\nint c;\n')  # a cycle ends
+    was = bench.source_digest(str(top))
+    deep.write_text('#include "sub/h.cuh"\nint c;  // note\n')
+    assert bench.source_digest(str(top)) == was
+    deep.write_text('#include "sub/h.cuh"\nint d;\n')
+    assert bench.source_digest(str(top)) != was
+
+
+def test_traffic_of_wide_blocks_is_unknown(monkeypatch):
+    """Cells with blocks of more than 16 AOs run another kernel too."""
+    src = os.path.join(bench.ROOT, "paper_2009_12505_gb300", "csrc", "hfx_zc.cu")
+    monkeypatch.setattr(bench, "ZC_CAPTURED_SHA", bench.source_digest(src))
+    assert bench.zc_traffic(1e12, 16) == bench.ZC_BYTES_PER_TENSOR_FLOP * 1e12
+    assert bench.zc_traffic(1e12, 17) is None
+
+
 def test_sample_atoms_and_term_total():
     assert bench.sample_atoms(8) == list(range(8))
     a = bench.sample_atoms(512)
