@@ -7,9 +7,10 @@ import ctypes
 import numpy as np
 import pytest
 
+import oracle
 import paper_2009_12505_gb300 as hfx
 import synth
-from gpu_common import gpu_build
+from gpu_common import compare_full, gpu_build
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -90,3 +91,13 @@ def test_split_after_fp64(workloads, nslices):
     ctx.set_blocks("C", b.C)
     ctx.build(THETA, "fp64")
     _same_as_fresh(b, ctx, "ozaki", nslices)
+
+
+@pytest.mark.parametrize("mode,tol", [(("fp64", 0), 1e-10), (("ozaki", 6), 1e-8)])
+def test_new_order_matches_oracle(workloads, mode, tol):
+    """C in the reverse order of size, set into a context that was built with the old order."""
+    a, b = workloads
+    ctx, _ = _context(a)
+    ctx.build(THETA, *mode)
+    ctx.set_blocks("C", b.C)
+    compare_full(b, THETA, gpu_build(b, THETA, *mode, ctx=ctx)[1], oracle.Oracle.of(b).build(THETA), tol)
