@@ -731,7 +731,8 @@ def run_gpu(args):
                                           "7-bit bf16 digits on tcgen05 (exact f32 group sums "
                                           "per digit order, added in int64 for D_AB and in "
                                           "double-float for Y, D_FG and D_FB); Y contraction "
-                                          "of the D_FG / D_FB pieces and P of the D_AB piece "
+                                          "of the D_FG / D_FB pieces (a second digit product for "
+                                          "blocks of more than 16 AOs) and P of the D_AB piece "
                                           "in double-float; Sigma in 128-bit fixed point")
                            if prec == "ozaki" else "FP64 CUDA cores; Sigma in 128-bit fixed point",
                            "l2": f"no flush: inputs {sum(getattr(wl, k).data.nbytes for k in 'CVD') / 1e9:.2f} GB per cell and GBs of per-wave scratch exceed the 129 MB L2",

@@ -48,7 +48,12 @@
  *                 straight to Sigma, and in double-float (f32 pairs, rounding
  *                 below the digit truncation) where it feeds a further
  *                 contraction (6 digits: about 41 significant bits per operand
- *                 row).
+ *                 row).  That contraction is in double-float too or, where a
+ *                 block or atom A has more than 16 NAOs, a second digit product
+ *                 of six 8-bit digits with an exponent per row and per output:
+ *                 it drops less than the first product did, in every element.
+ *                 P of the D_AB piece (an f32 pair) has each word rounded to
+ *                 the last digit's unit, ties to even.
  * Sigma is accumulated in 128-bit fixed point (integer adds, 2^-64 Ha
  * resolution) and converted to FP64 once, and E_X is summed from it in a
  * fixed order, so results are bitwise reproducible run to run in every mode.
@@ -148,6 +153,11 @@ hfx_status hfx_clear(hfx_ctx *ctx, char which);
  *   nslices  digits per operand: HFX_OZAKI 4..6 (0 = 6), HFX_BF16X3 0 or 2,
  *            HFX_FP64 ignored
  *   ex_out   receives E_X in Ha (host pointer), may be NULL
+ * Memory: the split modes keep C in three digit layouts beside the FP64 blocks,
+ * 2 nslices bytes per element each (plus padding to tiles); a fourth one when
+ * some atom has more than 16 NAOs (atoms of at most 16 are then held in both
+ * layouts of the D_FG / D_FB products).
+ * A failed call can be repeated: nothing that it left undone is taken as done.
  * Errors: HFX_E_STATE (no C, V or D set), HFX_E_ARG (also: a split mode with
  *         an atom of more than 32 NAOs), HFX_E_NOMEM, HFX_E_CUDA, HFX_E_TIMEOUT.
  */

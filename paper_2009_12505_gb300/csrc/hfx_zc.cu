@@ -53,7 +53,7 @@
 // operand reads.  In copies of the kernel on the 8-atom cell (25.7 ms), a quarter
 // of A's bytes changed nothing and no contraction at all took 18.3 ms; half the
 // contraction's arithmetic gained nothing either.  25.7 ms before the loader's lanes
-// and the contraction's unrolling, 22.4-23.2 ms now (7.2 ms of bf16 products).
+// and the contraction's unrolling, 21.9 ms now (7.2 ms of bf16 products).
 #include "zc_common.cuh"
 
 namespace split {

@@ -27,8 +27,8 @@
 // Roles (one CTA per SM, persistent): warps 0-15 as above; warp 16 streams A and
 // B tiles into a ring of shared stages, warp 17 issues the tcgen05 MMAs into one
 // of two TMEM accumulators, warp 18 copies each tile's Y rows and row
-// exponents.  Every wait is bounded; on expiry the kernel records HFX_DEV_ERR_TIMEOUT, drains its copies and MMAs,
-// frees TMEM and returns.
+// exponents.  Every wait is bounded; on expiry the kernel records
+// HFX_DEV_ERR_TIMEOUT, drains its copies and MMAs, frees TMEM and returns.
 //
 // What bounds it: the epilogue, beside up to 22 operand stages a tile.  8-atom
 // two-element cell (13/60 and 27/90, C, D to 9 bohr): 178.7 ms for its wide jobs
